@@ -6,6 +6,7 @@
 #include <new>
 #include <vector>
 #include "internal.cuh"
+#include "digit.cuh"
 #include "fft_fixed.cuh"
 #include "solve.cuh"
 
@@ -136,6 +137,8 @@ void free_ctx(rfnse_ctx* c) {
   cudaFree(c->adj_red);
   for (int a = 0; a < 3; ++a) {
     cudaFree(c->twdf[a]);
+    cudaFree(c->digS[a]);
+    cudaFree(c->digT[a]);
     for (int h = 0; h < 2; ++h) cudaFree(c->circdf[h][a]);
   }
   for (int a = 0; a < 3; ++a) {
@@ -287,6 +290,14 @@ int rfnse_create(const rfnse_params* p, void* stream, rfnse_ctx** out) {
       }
     }
   }
+  if (c->d > 1)  // digit passes of the axes that have them
+    for (int a = 0; a < c->d; ++a) {
+      DigitShape sh;
+      if (!digit_shape(c->n[a], &sh)) continue;
+      chk(dev_alloc(&c->digS[a], digit_table_bytes(sh)));
+      chk(dev_alloc(&c->digT[a], digit_table_bytes(sh)));
+      c->digT_exp[a] = digit_exp_toeplitz(p->alpha, c->mu[a]);
+    }
   c->red_blocks = choose_reduce_blocks(N);
   {
     const char* dbg = std::getenv("RFNSE_DEBUG");
@@ -320,6 +331,10 @@ int rfnse_create(const rfnse_params* p, void* stream, rfnse_ctx** out) {
   launch_setup_coefficients(c->c, nmax, p->alpha, c->stream);
   for (int a = 0; a < c->d; ++a) {
     launch_setup_axis(c->c, c->n[a], c->L[a], c->lam[a], c->circ[a], c->tw64[a], c->tw32[a], c->stream);
+    if (c->digS[a]) {
+      launch_setup_digits(c->c, c->n[a], 1.0, 0, digit_exp_dst(c->n[a]), a == 0, c->digS[a], c->stream);
+      launch_setup_digits(c->c, c->n[a], c->mu[a], 1, c->digT_exp[a], a == 0, c->digT[a], c->stream);
+    }
     if (p->precond == 1)
       launch_setup_circ(c->c, c->n[a], c->L[a], c->lamC[a], c->chirp64[a], c->chirp32[a], c->bspec64[a],
                         c->bspec32[a], c->stream);

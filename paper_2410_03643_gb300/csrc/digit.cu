@@ -1,0 +1,565 @@
+// The FP64 digit-pass kernel and its launches (see digit.cuh).
+#include <cuda_fp16.h>
+#include <cmath>
+#include "digit.cuh"
+#include "tc05.cuh"
+
+namespace rfnse {
+
+namespace {
+
+struct DigitArgs {
+  const unsigned char* table;  // operator digits (k_digit_table)
+  int oexp;                    // operator entry = integer * 2^oexp
+  int log2N, stack;            // log2(n + 1), lines stacked in one column
+  int ca_code, cb_code;        // ca, cb as in the double-float passes (-1: any value)
+  double lam_scale;            // 1 / dst_scale: lamfac holds i dst_scale / (omega + i Lambda)
+  int* err;                    // set when a bounded wait gives up
+};
+
+// Shared memory: barriers and line exponents, the vector's digits, the chunk ring.  The digits are one
+// K-major operand of 224 columns, digit j of column n at 32 j + n, because D_i .. D_6 are neighbours in
+// TMEM: for one operator digit a_i a single MMA of N = 32 (7 - i) columns forms its products with x_0 ..
+// x_{6-i}.  (An MMA costs 44 + N/2 cycles with A in shared memory, measured for N = 16..128: seven MMAs of
+// 32..224 columns per 16 entries take 751 cycles, 28 of 32 columns 1680.)  Core matrices lie 128 B (next
+// 8 columns) and 3616 B (next 8 entries) apart, so that both the threads of a strided pass (neighbouring
+// columns) and of an x pass (neighbouring entries, real and imaginary column) store without bank conflicts.
+constexpr int kSbo = 128, kLbo = kDigits * (kDigCols / 8) * kSbo + 32;
+constexpr int kDigitPitch = (kDigCols / 8) * kSbo;  // bytes from a digit to the next
+constexpr int kCtrl = 1024;
+constexpr int kRowPitch = kDigLines * 16 + 16;  // staged results: a row's 16 lines, 16 B each
+template <int KB> constexpr int digit_bytes() { return (16 * KB * kLbo + 127) & ~127; }
+template <int KB> constexpr int digit_smem() { return kCtrl + digit_bytes<KB>() + kDigStages * kDigChunkBytes; }
+
+// x as a fixed-point integer on the scale of exponent emax: |X| < 2^61, x = X 2^(emax - 1083)
+__device__ __forceinline__ long long to_fixed(double x, int emax) {
+  const int hi = __double2hiint(x);
+  const unsigned lo = (unsigned)__double2loint(x);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned mh = ((unsigned)hi & 0xfffffu) | (e ? 0x100000u : 0u);
+  const int sh = emax - (e ? e : 1);
+  unsigned long long m = (((unsigned long long)mh << 32) | lo) << 8;
+  m = sh > 63 ? 0ull : m >> sh;
+  return hi < 0 ? -(long long)m : (long long)m;
+}
+
+// v 2^ex rounded to nearest (truncated below the normal range, infinity above it)
+__device__ __forceinline__ double from_fixed(long long v, int ex) {
+  const unsigned long long m = v < 0 ? 0ull - (unsigned long long)v : (unsigned long long)v;
+  if (m == 0) return 0.0;
+  const int lz = __clzll((long long)m);
+  const unsigned long long t = m << lz;
+  const unsigned long long r = (t >> 11) + ((t >> 10) & 1);  // 2^52 .. 2^53
+  const int E = ex + 63 - lz + 1023;
+  unsigned long long b = E <= 0 ? (E < -60 ? 0ull : r >> (1 - E))
+                         : E >= 2047 ? 0x7ff0000000000000ull
+                                     : ((unsigned long long)(E - 1) << 52) + r;
+  b |= (unsigned long long)v & 0x8000000000000000ull;
+  return __longlong_as_double((long long)b);
+}
+
+__device__ __forceinline__ uint32_t half2_sub(uint32_t a, uint32_t b) {
+  const __half2 r = __hsub2(*reinterpret_cast<const __half2*>(&a), *reinterpret_cast<const __half2*>(&b));
+  return *reinterpret_cast<const uint32_t*>(&r);
+}
+
+// The seven digits of two fixed-point values, packed as FP16 pairs: digit i of Y (biased so that every
+// field is unsigned) is put below the exponent of 1024, whose ulp is one unit, and the offset subtracted.
+__device__ __forceinline__ void digits2(long long y0, long long y1, uint32_t (&d)[kDigits]) {
+  constexpr long long bias = 0x4020100804020100ll;  // 256 (1 + 2^9 + ... + 2^54)
+  const unsigned long long a = (unsigned long long)(y0 + bias), b = (unsigned long long)(y1 + bias);
+#pragma unroll
+  for (int i = 0; i < kDigits; ++i) {
+    const uint32_t fa = (uint32_t)(a >> (54 - 9 * i)), fb = (uint32_t)(b >> (54 - 9 * i));
+    const uint32_t f = __byte_perm(fa, fb, 0x5410) & (i == 0 ? 0x03ff03ffu : 0x01ff01ffu);
+    d[i] = half2_sub(f | 0x64006400u, 0x65006500u);
+  }
+}
+
+__device__ __forceinline__ double2 coef_times(int code, double2 c, double2 v) {
+  switch (code) {
+    case 0: return make_double2(0.0, 0.0);
+    case 1: return v;
+    case 2: return make_double2(-v.x, -v.y);
+    case 3: return make_double2(-v.y, v.x);
+    case 4: return make_double2(v.y, -v.x);
+    default: return cmul(c, v);
+  }
+}
+
+// KB: K / 128 of a half; FOLD: sums and differences (two halves), else stacked whole lines.
+template <int FLAGS, int KB, bool FOLD>
+__global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassParams p, const DigitArgs a) {
+  constexpr bool TOEP = (FLAGS & (F_TOEP_X | F_TOEP_ACC)) != 0;
+  constexpr bool PAIR = FOLD && TOEP;  // both halves of a result are needed: a cluster of two blocks
+  constexpr int NT = 512 * KB;
+  constexpr int NK = 128 * KB / kDigChunkK;  // chunks per operator digit
+  constexpr int NC = kDigits * NK;
+  constexpr uint32_t COLS = KB == 1 ? 256 : 512;
+  if (p.skip && *p.skip) return;  // uniform over the launch
+  extern __shared__ __align__(128) unsigned char sm[];
+  unsigned char* dig = sm + kCtrl;
+  const uint32_t s0 = tc::smem_addr(sm), sdig = s0 + kCtrl;
+  const uint32_t sring = sdig + digit_bytes<KB>();
+  const uint32_t b_full = s0, b_empty = s0 + 8 * kDigStages, b_done = s0 + 16 * kDigStages;
+  uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + 96);
+  int* s_fail = reinterpret_cast<int*>(sm + 100);
+  unsigned* smax = reinterpret_cast<unsigned*>(sm + 128);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+
+  int h = 0, mb = 0;
+  long long tile = blockIdx.x;
+  if (FOLD) {
+    h = (int)(tile & 1);
+    tile >>= 1;
+    if (KB == 2) {
+      mb = (int)(tile & 1);
+      tile >>= 1;
+    }
+  }
+  const unsigned char* tab = a.table + ((size_t)h * KB + mb) * NC * kDigChunkBytes;
+
+  if (warp == 0) {
+    if (lane == 0) {
+      for (int i = 0; i < kDigStages; ++i) {
+        tc::mbar_init(b_full + 8 * i, 1);
+        tc::mbar_init(b_empty + 8 * i, 1);
+      }
+      tc::mbar_init(b_done, 1);
+      tc::mbar_init_fence();
+      *s_fail = 0;
+    }
+    if (lane < kDigLines) smax[lane] = 0;
+    __syncwarp();
+    tc::tmem_alloc(tc::smem_addr(s_tmem), COLS);
+    tc::fence_before();
+  }
+  __syncthreads();
+  tc::fence_after();
+  const uint32_t tmem = *s_tmem;
+  auto load_chunk = [&](int c) {
+    const int st = c % kDigStages;
+    tc::mbar_expect_tx(b_full + 8 * st, kDigChunkBytes);
+    tc::bulk_load(sring + st * kDigChunkBytes, tab + (size_t)c * kDigChunkBytes, kDigChunkBytes, b_full + 8 * st);
+  };
+  if (tid == 32)
+    for (int c = 0; c < kDigStages; ++c) load_chunk(c);
+
+  // ---- this thread's eight entries (and their mirror images) of one column: the real or the imaginary
+  // part of a line, neighbouring lanes of a warp, so that a warp reads 256 consecutive bytes -------------
+  const bool xax = p.stride == 1;
+  const int n = p.n;
+  const int part = tid & 1, t16 = (tid >> 1) & 15;
+  const int l = xax ? ((tid >> 5) & 15) : t16;
+  const int kg = xax ? ((tid >> 9) * 16 + t16) : (tid >> 5);
+  auto slot_pos = [&](int i) { return xax ? (kg >> 4) * 128 + i * 16 + t16 : kg * 8 + i; };
+  const long long hi = xax ? 0 : tile / p.tiles_inner;
+  const long long line0 = xax ? tile * (kDigLines * a.stack) : (tile - hi * p.tiles_inner) * (kDigLines * a.stack);
+  const long long nline = xax ? p.nlines : p.stride;       // lines that line0 + ... runs over
+  const long long base0 = xax ? 0 : hi * p.stride * n;
+  const long long lstep = xax ? n : 1, estep = xax ? 1 : p.stride;
+
+  double va[8];
+  [[maybe_unused]] double vb[8];
+  {
+    const double2* in = reinterpret_cast<const double2*>(p.in);
+    double2* cpy = p.copy_out;
+    double sc = 1.0;
+    if constexpr ((FLAGS & F_INSCALE) != 0) {
+      if (p.gdyn) {
+        in = p.gdyn->src;
+        sc = p.gdyn->src_scale;
+        cpy = p.vbase + (long long)p.gdyn->j * p.ldv;
+      } else {
+        sc = *p.in_scale;
+      }
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const int q = slot_pos(i);
+      va[i] = 0.0;
+      if constexpr (FOLD) {
+        vb[i] = 0.0;
+        if (line0 + l < nline) {
+          const double* s = reinterpret_cast<const double*>(in + base0 + (line0 + l) * lstep) + part;
+          va[i] = s[2 * (q * estep)];
+          if (2 * q != n - 1) vb[i] = s[2 * ((n - 1 - q) * estep)];
+        }
+      } else {
+        const int sl = q >> a.log2N, pos = q - (sl << a.log2N);
+        const long long ln = line0 + sl * kDigLines + l;
+        if (ln < nline && pos < n) va[i] = reinterpret_cast<const double*>(in + base0 + ln * lstep + pos * estep)[part];
+      }
+    }
+    if constexpr ((FLAGS & F_INSCALE) != 0) {
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int q = slot_pos(i);
+        va[i] *= sc;
+        if constexpr (FOLD) {
+          vb[i] *= sc;
+          if (h == 0 && mb == 0 && line0 + l < nline) {
+            double* d = reinterpret_cast<double*>(cpy + base0 + (line0 + l) * lstep) + part;
+            d[2 * (q * estep)] = va[i];
+            if (2 * q != n - 1) d[2 * ((n - 1 - q) * estep)] = vb[i];
+          }
+        } else {
+          const int sl = q >> a.log2N, pos = q - (sl << a.log2N);
+          const long long ln = line0 + sl * kDigLines + l;
+          if (ln < nline && pos < n) reinterpret_cast<double*>(cpy + base0 + ln * lstep + pos * estep)[part] = va[i];
+        }
+      }
+    }
+  }
+  {  // the column's largest exponent
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      m = max(m, (unsigned)__double2hiint(va[i]) & 0x7fffffffu);
+      if constexpr (FOLD) m = max(m, (unsigned)__double2hiint(vb[i]) & 0x7fffffffu);
+    }
+    if (xax) {
+      m = __reduce_max_sync(0xffffffffu, m);
+      if (lane == 0) atomicMax(&smax[l], m);
+    } else {
+      m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+      if (part == 0) atomicMax(&smax[l], m);
+    }
+  }
+  __syncthreads();
+  {
+    const int emax = max((int)(smax[l] >> 20), 1);
+    const int col = 2 * l + part;
+    unsigned char* dst = dig + kg * kLbo + (col >> 3) * kSbo + (col & 7) * 16;
+    uint32_t w[kDigits][4];
+#pragma unroll
+    for (int i = 0; i < 8; i += 2) {
+      long long y[2];
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        y[k] = to_fixed(va[i + k], emax);
+        if constexpr (FOLD) {
+          const long long m = to_fixed(vb[i + k], emax);
+          if (h == 0) y[k] += m;
+          else y[k] = 2 * slot_pos(i + k) != n - 1 ? y[k] - m : 0;
+        }
+      }
+      uint32_t d[kDigits];
+      digits2(y[0], y[1], d);
+#pragma unroll
+      for (int j = 0; j < kDigits; ++j) w[j][i >> 1] = d[j];
+    }
+#pragma unroll
+    for (int j = 0; j < kDigits; ++j)
+      *reinterpret_cast<uint4*>(dst + j * kDigitPitch) = make_uint4(w[j][0], w[j][1], w[j][2], w[j][3]);
+  }
+  tc::fence_async_smem();
+  __syncthreads();
+
+  // ---- products: one warp issues the MMAs (all its values warp-uniform: an MMA issued from a divergent
+  // branch costs 125 cycles or more of issue), another refills the chunk ring --------------------------
+  int issued = kDigStages;  // chunks requested so far (warp 1)
+  const int uwarp = __shfl_sync(0xffffffffu, warp, 0);
+  if (uwarp == 0) {
+    tc::fence_after();
+    const bool one = tc::elect_one();
+    const uint32_t ud = __shfl_sync(0xffffffffu, tmem, 0);
+    const uint64_t da0 = tc::smem_desc(__shfl_sync(0xffffffffu, sring, 0), 2048, 128);
+    const uint64_t db0 = tc::smem_desc(__shfl_sync(0xffffffffu, sdig, 0), kLbo, kSbo);
+    bool ok = true;
+    int st = 0, ph = 0;
+    for (int i = 0; i < kDigits && ok; ++i) {
+      const uint32_t id = tc::idesc_f16(128, kDigCols * (kDigits - i));
+      for (int kc = 0; kc < NK; ++kc) {
+        ok = tc::mbar_wait(b_full + 8 * st, ph);
+        if (!ok) break;
+        const uint32_t kb = KB == 1 ? 0 : (uint32_t)kc / (128 / kDigChunkK);
+        const uint32_t d = ud + (kb * kDigits + i) * kDigCols;
+        const bool first = i == 0 && kc % (128 / kDigChunkK) == 0;
+#pragma unroll
+        for (int ks = 0; ks < kDigChunkK / 16; ++ks) {
+          const uint64_t da = da0 + (uint32_t)((st * kDigChunkBytes + ks * 4096) >> 4);
+          const uint64_t db = db0 + (uint32_t)(((kc * (kDigChunkK / 16) + ks) * 2 * kLbo) >> 4);
+          if (one) tc::mma_f16(d, da, db, id, !(first && ks == 0));
+        }
+        if (one) tc::mma_commit(b_empty + 8 * st);
+        if (++st == kDigStages) {
+          st = 0;
+          ph ^= 1;
+        }
+      }
+    }
+    if (one) tc::mma_commit(b_done);
+    if (!ok && lane == 0) *s_fail = 1;
+  } else if (uwarp == 1) {
+    for (int c = kDigStages; c < NC; ++c) {
+      if (!tc::mbar_wait(b_empty + 8 * (c % kDigStages), ((c / kDigStages) & 1) ^ 1)) {
+        if (lane == 0) *s_fail = 1;
+        break;
+      }
+      if (lane == 0) load_chunk(c);
+      issued = c + 1;
+    }
+  }
+  __syncwarp();
+  if (!tc::mbar_wait(b_done, 0)) *s_fail = 1;
+  tc::fence_after();
+  __syncthreads();
+  if (*s_fail) {  // uniform: a wait gave up; wait for the copies in flight, free TMEM and leave
+    if (tid == 32) {
+      for (int c = issued - kDigStages; c < issued; ++c)
+        tc::mbar_wait(b_full + 8 * (c % kDigStages), (c / kDigStages) & 1);
+      if (a.err) *(volatile int*)a.err = 1;
+    }
+    __syncthreads();
+    if (warp == 0) tc::tmem_free(tmem, COLS);
+    if constexpr (PAIR) {
+      tc::cluster_sync();
+      tc::cluster_sync();
+    }
+    return;
+  }
+
+  // ---- accumulators -> 64-bit integers, staged by row (over the digits, which the MMAs have read) --------
+  {
+    constexpr int CW = kDigCols / (4 * KB);  // columns of this warp
+    constexpr int SH = TOEP ? kDigShiftT : kDigShiftS;
+    const int row = 32 * (warp & 3) + lane;
+#pragma unroll
+    for (int c0 = (warp >> 2) * CW, b = 0; b < CW / 4; ++b, c0 += 4) {
+      const uint32_t ta = tmem + ((uint32_t)(32 * (warp & 3)) << 16) + (uint32_t)c0;
+      long long v[4];
+#pragma unroll
+      for (int kb = 0; kb < KB; ++kb) {
+        float D[kDigits][4];
+#pragma unroll
+        for (int d = 0; d < kDigits; ++d) tc::tmem_ld(ta + (kb * kDigits + d) * kDigCols, D[d]);
+        tc::tmem_ld_wait(D);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {  // sum_d D_d 2^(SH - 9d)
+          const long long up = (long long)__float2int_rn(D[0][i]) * 262144 +
+                               ((long long)__float2int_rn(D[1][i]) * 512 + __float2int_rn(D[2][i]));
+          const long long mid = (long long)__float2int_rn(D[3][i]) * 512 + __float2int_rn(D[4][i]);
+          const int low = __float2int_rn(fmaf(D[6][i], 0x1p-9f, D[5][i]) * (TOEP ? 1.0f : 0x1p-5f));
+          const long long s = (up << (SH - 18)) + (mid << (SH - 36)) + low;
+          v[i] = kb ? v[i] + s : s;
+        }
+      }
+      unsigned char* dst = dig + row * kRowPitch + (c0 >> 1) * 16;
+#pragma unroll
+      for (int i = 0; i < 4; i += 2)
+        *reinterpret_cast<longlong2*>(dst + (i >> 1) * 16) = make_longlong2(v[i], v[i + 1]);
+    }
+  }
+  tc::fence_before();
+  __syncthreads();
+  if (warp == 0) {
+    tc::fence_after();
+    tc::tmem_free(tmem, COLS);
+  }
+  if constexpr (PAIR) tc::cluster_sync();
+
+  // ---- results: convert and apply the pass's pointwise work, in grid order -------------------------------
+  [[maybe_unused]] double dot = 0.0, nrm = 0.0;
+  const double nan = __longlong_as_double(0x7ff8000000000000ll);
+  struct Operands {
+    double2 u, z, acc;
+    double D;
+  };
+  [[maybe_unused]] double2* zout = reinterpret_cast<double2*>(p.out);
+  auto fetch = [&](long long g, bool ok) {
+    Operands o;
+    o.u = o.z = o.acc = make_double2(0.0, 0.0);
+    o.D = 0.0;
+    if (!ok) return o;
+    if constexpr ((FLAGS & F_LAM) != 0) o.u = reinterpret_cast<const double2*>(p.lamfac)[g];
+    if constexpr ((FLAGS & F_DSCALE) != 0) {
+      o.u = reinterpret_cast<const double2*>(p.dfac)[g];
+      if (p.z_add) o.acc = zout[g];
+    }
+    if constexpr (TOEP) {
+      if (p.acc_in) o.acc = reinterpret_cast<const double2*>(p.acc_in)[g];
+      if constexpr ((FLAGS & F_TOEP_X) != 0) {
+        o.z = reinterpret_cast<const double2*>(p.in)[g];
+        if (p.Dr) o.D = reinterpret_cast<const double*>(p.Dr)[g];
+      }
+      if constexpr ((FLAGS & F_DOT0) != 0) o.u = p.dot_v0[g];
+    }
+    return o;
+  };
+  auto emit = [&](long long g, long long re, long long im, int ln, const Operands& o) {
+    const int emax = (int)(smax[ln] >> 20);
+    const int ex = max(emax, 1) - 975 - (TOEP ? kDigShiftT : kDigShiftS) + a.oexp;
+    double2 y = make_double2(from_fixed(re, ex), from_fixed(im, ex));
+    if (emax == 2047) y = make_double2(nan, nan);  // an infinity or NaN on the line
+    if constexpr ((FLAGS & F_DST) != 0 && (FLAGS & F_DSCALE) == 0) {
+      if constexpr ((FLAGS & F_LAM) != 0) {
+        y = cmul(y, o.u);
+        y = make_double2(y.y * a.lam_scale, -y.x * a.lam_scale);
+      }
+      reinterpret_cast<double2*>(p.out)[g] = y;
+    }
+    if constexpr ((FLAGS & F_DSCALE) != 0) {
+      y = cmul(y, o.u);
+      zout[g] = p.z_add ? cadd(o.acc, y) : y;
+    }
+    if constexpr (TOEP) {
+      double2 acc = o.acc;
+      if constexpr ((FLAGS & F_TOEP_X) != 0) {
+        if (p.Dr) {
+          y.x = fma(-o.D, o.z.x, y.x);
+          y.y = fma(-o.D, o.z.y, y.y);
+        }
+        if (a.ca_code != 0) acc = cadd(acc, coef_times(a.ca_code, p.ca, o.z));
+      }
+      acc = cadd(acc, coef_times(a.cb_code, p.cb, y));
+      reinterpret_cast<double2*>(p.acc_out)[g] = acc;
+      if constexpr ((FLAGS & F_DOT0) != 0) {
+        dot = fma(o.u.x, acc.x, dot);
+        dot = fma(o.u.y, acc.y, dot);
+      }
+      if (p.nrm_part) {
+        nrm = fma(acc.x, acc.x, nrm);
+        nrm = fma(acc.y, acc.y, nrm);
+      }
+    }
+  };
+  if constexpr (PAIR) {  // y_j = e_j + o_j, y_{N-j} = e_j - o_j; this block finishes eight of the lines
+    constexpr int ITEMS = 128 * 8 / NT;
+#pragma unroll 2
+    for (int it = 0; it < ITEMS; ++it) {
+      const int e = it * NT + tid;
+      const int r = xax ? (e & 127) : (e >> 3), ln = 8 * h + (xax ? (e >> 7) : (e & 7));
+      const int q = mb * 128 + r;
+      const bool ok = line0 + ln < nline, two = 2 * q != n - 1;
+      const long long g = base0 + (line0 + ln) * lstep + q * estep;
+      const long long g2 = base0 + (line0 + ln) * lstep + (n - 1 - q) * estep;
+      const Operands o1 = fetch(g, ok), o2 = fetch(g2, ok && two);
+      const uint32_t at = sdig + r * kRowPitch + ln * 16;
+      long long er, ei, dr, di;
+      tc::ld_cluster(at, 0, er, ei);
+      tc::ld_cluster(at, 1, dr, di);
+      if (ok) emit(g, er + dr, ei + di, ln, o1);
+      if (ok && two) emit(g2, er - dr, ei - di, ln, o2);
+    }
+    tc::cluster_sync();
+  } else {
+    constexpr int ITEMS = 128 * kDigLines / NT;
+#pragma unroll 2
+    for (int it = 0; it < ITEMS; ++it) {
+      const int e = it * NT + tid;
+      const int r = xax ? (e & 127) : (e >> 4), ln = xax ? (e >> 7) : (e & 15);
+      int pos;
+      long long line = line0 + ln;
+      if constexpr (FOLD) {
+        pos = 2 * (mb * 128 + r) + h;
+      } else {
+        const int sl = r >> a.log2N;
+        pos = r - (sl << a.log2N);
+        line += sl * kDigLines;
+      }
+      const bool ok = line < nline && pos < n;
+      const long long g = base0 + line * lstep + pos * estep;
+      const Operands o = fetch(g, ok);
+      const longlong2 v = *reinterpret_cast<const longlong2*>(dig + r * kRowPitch + ln * 16);
+      if (ok) emit(g, v.x, v.y, ln, o);
+    }
+  }
+  if constexpr ((FLAGS & F_DOT0) != 0) block_sum_store(dot, p.dot_part + blockIdx.x);
+  if constexpr (TOEP)
+    if (p.nrm_part) block_sum_store(nrm, p.nrm_part + blockIdx.x);
+}
+
+int coef_code(double2 c) {
+  if (c.x == 0.0 && c.y == 0.0) return 0;
+  if (c.x == 1.0 && c.y == 0.0) return 1;
+  if (c.x == -1.0 && c.y == 0.0) return 2;
+  if (c.x == 0.0 && c.y == 1.0) return 3;
+  if (c.x == 0.0 && c.y == -1.0) return 4;
+  return -1;
+}
+
+template <int FLAGS, int KB, bool FOLD>
+cudaError_t launch_digit(const PassParams& p, const DigitArgs& a, unsigned grid, cudaStream_t s) {
+  auto kern = k_digit<FLAGS, KB, FOLD>;
+  constexpr int smem = digit_smem<KB>();
+  static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (attr != cudaSuccess) return attr;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(grid);
+  cfg.blockDim = dim3(512 * KB);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  if (FOLD && (FLAGS & (F_TOEP_X | F_TOEP_ACC))) {
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+  }
+  count_launch();
+  return cudaLaunchKernelEx(&cfg, kern, p, a);
+}
+
+}  // namespace
+
+bool digit_possible(const rfnse_ctx* c, int axis) { return c->digS[axis] != nullptr; }
+
+// A single tile takes 8 us whatever its size, and a fused FFT pass is two launches here: below 8192 points
+// the FFT passes are as fast or faster (63 x 31: 15.4 / 24.0 us for S / T along x against 14.5 / 16.0 here,
+// but 15.4 against 29 for the fused pair), from 127^2 on these are (127^2: S 17.8 and 23.5 us along x and y
+// against 15; 511^2: 47 against 24, T 87 against 27; 255^3: S 2000 against 415, T 3870 against 475).
+bool digit_pays(const rfnse_ctx* c, int axis) { return c->N >= 8192 && digit_possible(c, axis); }
+
+template <int FLAGS>
+cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s) {
+  constexpr bool TOEP = (FLAGS & (F_TOEP_X | F_TOEP_ACC)) != 0;
+  DigitShape sh;
+  if (!digit_possible(c, axis) || !digit_shape(p.n, &sh)) return cudaErrorInvalidValue;
+  DigitArgs a{};
+  a.table = static_cast<const unsigned char*>(TOEP ? c->digT[axis] : c->digS[axis]);
+  a.oexp = TOEP ? c->digT_exp[axis] - (half ? 1 : 0) : digit_exp_dst(p.n);
+  a.log2N = p.log2L - 1;
+  a.stack = sh.stack;
+  a.ca_code = coef_code(p.ca);
+  a.cb_code = coef_code(p.cb);
+  a.lam_scale = 1.0 / p.dst_scale;
+  a.err = &c->gs->err;
+  const long long per = (long long)kDigLines * sh.stack;
+  long long tiles;
+  if (p.stride == 1) {
+    p.tiles_inner = 1;
+    tiles = (p.nlines + per - 1) / per;
+  } else {
+    p.tiles_inner = (p.stride + per - 1) / per;
+    tiles = p.tiles_inner * (p.nlines / p.stride);
+  }
+  const long long grid = tiles * sh.halves * sh.kb;
+  if (grid <= 0) return cudaSuccess;
+  if constexpr ((FLAGS & F_DOT0) != 0) {  // too many partials for the Arnoldi kernel to sum: plain pass
+    if (grid > kDot0MaxBlocks) {
+      c->dot0_blocks = 0;
+      return run_digit<(FLAGS & ~F_DOT0)>(c, p, axis, half, s);
+    }
+    c->dot0_blocks = (int)grid;
+  }
+  if (p.nrm_part) {
+    if (grid > kNormPartMax) p.nrm_part = nullptr;
+    c->nrm_df_blocks = p.nrm_part ? (int)grid : 0;
+  }
+  if (sh.halves == 1) return launch_digit<FLAGS, 1, false>(p, a, (unsigned)grid, s);
+  if (sh.kb == 1) return launch_digit<FLAGS, 1, true>(p, a, (unsigned)grid, s);
+  return launch_digit<FLAGS, 2, true>(p, a, (unsigned)grid, s);
+}
+
+#define RFNSE_DIGIT(F) template cudaError_t run_digit<F>(rfnse_ctx*, PassParams, int, int, cudaStream_t);
+RFNSE_DIGIT(F_INSCALE | F_DST)
+RFNSE_DIGIT(F_DST)
+RFNSE_DIGIT(F_DST | F_LAM)
+RFNSE_DIGIT(F_DST | F_DSCALE)
+RFNSE_DIGIT(F_TOEP_X)
+RFNSE_DIGIT(F_TOEP_ACC)
+RFNSE_DIGIT(F_TOEP_ACC | F_DOT0)
+
+}  // namespace rfnse

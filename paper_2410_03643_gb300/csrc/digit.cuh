@@ -1,0 +1,190 @@
+// Digit passes: a transform along one grid axis (the DST-I S, or the Toeplitz product mu_a T_0) as a
+// dense product on the tensor cores, exact to FP64 rounding.  GB300 issues two FP64 FMAs per SM and
+// cycle, 1/61 of its FP32 rate, so an FP64 FFT pass is bound by that pipe; a tensor-core product of
+// FP16 digits is not.
+//
+// Every line is scaled by a power of two to a fixed-point integer, X = sum_i x_i 2^(54 - 9i) with seven
+// balanced digits |x_i| <= 256; the operator's entries likewise, A = sum_i a_i 2^(54 - 9i), |a_0| <= 128,
+// tabulated at set-up.  Digits are FP16 operands of tcgen05.mma with FP32 accumulators in TMEM.  The
+// products of one weight, D_d = sum_{i + j = d} sum_k a_i[r,k] x_j[k] over 128 entries k, are integers below
+// 2^24 (a row's lower digits average 128: 2^22 per product), so the FP32 sums of the leading weights are exact;
+// d = 0..6 are formed, 28 products, and combined in 64-bit integers.  What is dropped is 2^-61 of a line's
+// largest entry times the operator's largest; the roundings left are those of the tabulated entries, of the
+// integer sum and of the conversion to double.  On random and on smooth lines of 3 to 511 points the
+// result is as near the exact product as an FP64 FFT's or nearer (two digits less would not be: the Toeplitz
+// product of a smooth line cancels to 10^-3 of its terms).
+//
+// Both operators commute with the reflection j -> N - j of a line (N = n + 1, up to the parity of the
+// sine mode), so for n >= 255 a line is folded into its sums s_j = x_j + x_{N-j} (with x_{N/2}) and
+// differences d_j = x_j - x_{N-j}, and each half is a product of size N/2: half the work.  Shorter
+// lines are not folded; 128 / N of them are stacked into one column of 128 entries and the operator is
+// block diagonal.
+//
+// Tile of a block: 128 operator rows of one half (all of it for n <= 255) times 32 columns (the real and
+// imaginary parts of 16 lines).
+#pragma once
+#include <cstdint>
+#include "internal.cuh"
+#include "passes.cuh"
+
+namespace rfnse {
+
+constexpr int kDigits = 7;        // digits of an entry = accumulators (weights) per output
+// result = sum_d D_d 2^(shift - 9d) in 64 bits: |D_0| < 2^17 for the Toeplitz rows (sum |c_k| = 2 c_0), and
+// < 2^23 for the sine rows of two 128-entry blocks
+constexpr int kDigShiftT = 45, kDigShiftS = 40;
+constexpr int kDigCols = 32;      // columns of a tile: 16 lines, real and imaginary part
+constexpr int kDigLines = 16;
+constexpr int kDigChunkK = 32;    // operator entries along K per chunk: 128 rows x 32 x 2 B = 8 KB
+constexpr int kDigChunkBytes = 128 * kDigChunkK * 2;
+constexpr int kDigStages = 5;     // chunks in flight
+
+// Geometry of an axis of n points: K/128 per half, halves, lines stacked in one column.
+struct DigitShape {
+  int kb, halves, stack;
+};
+inline bool digit_shape(int n, DigitShape* s) {
+  const int N = n + 1;
+  if (N <= 128) *s = {1, 1, 128 / N};
+  else if (N == 256) *s = {1, 2, 1};
+  else if (N == 512) *s = {2, 2, 1};
+  else return false;
+  return true;
+}
+// bytes of an operator's digit table: halves x row blocks x digits x K/32 chunks
+inline size_t digit_table_bytes(const DigitShape& s) {
+  return (size_t)s.halves * s.kb * kDigits * (s.kb * 128 / kDigChunkK) * kDigChunkBytes;
+}
+
+// The operator tables of one axis (set-up): S and mu_a T_0, each value = integer * 2^exp.
+// entry = 0: the DST-I, 1: the Toeplitz operator (coefficients c scaled by mu)
+void launch_setup_digits(const double* c, int n, double mu, int toeplitz, int exp, bool xax, void* table,
+                         cudaStream_t s);
+// exponent e with every |entry| <= 2^(e + 61)
+int digit_exp_dst(int n);
+int digit_exp_toeplitz(double alpha, double mu);
+
+// Whether the FP64 passes of an axis run as digit passes by default, whether they can, and one digit pass:
+// all storage FP64, FLAGS as for the line passes with one transform ([F_INSCALE |] F_DST, F_DST | F_LAM =
+// S x / (omega + i Lambda), F_DST | F_DSCALE, F_TOEP_X, F_TOEP_ACC [| F_DOT0]); half: the first step's mu_a / 2.
+bool digit_pays(const rfnse_ctx* c, int axis);
+bool digit_possible(const rfnse_ctx* c, int axis);
+template <int FLAGS>
+cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s);
+
+// The passes that have a digit form: FP64 throughout, a sine transform or a Toeplitz product, and not the
+// fused pass of 1-D grids (one launch there, three as digit passes).
+template <typename R, typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
+constexpr bool digit_form() {
+  return sizeof(R) == 8 && sizeof(TIN) == 16 && sizeof(TOUT) == 16 && sizeof(TACCI) == 16 && sizeof(TACCO) == 16 &&
+         !(FLAGS & F_CIRC) && ((FLAGS & F_DST) || !(FLAGS & F_DSCALE)) && !((FLAGS & F_LAM) && (FLAGS & F_DSCALE));
+}
+
+// CUDA events around the launches of a profiled pass (rfnse_profile): the stop event, null when the pass
+// is not of the profiled kind.
+template <int KIND>
+cudaError_t prof_start(rfnse_ctx* c, cudaStream_t s, cudaEvent_t* stop) {
+  *stop = nullptr;
+  if (c->prof_kind == 0 || (c->prof_kind | F_INSCALE | F_DOT0) != (KIND | F_INSCALE | F_DOT0)) return cudaSuccess;
+  while (c->prof_used + 2 > c->prof_events.size()) {
+    cudaEvent_t ev;
+    const cudaError_t e = cudaEventCreate(&ev);
+    if (e != cudaSuccess) return e;
+    c->prof_events.push_back(ev);
+  }
+  *stop = c->prof_events[c->prof_used + 1];
+  const cudaError_t e = cudaEventRecord(c->prof_events[c->prof_used], s);
+  c->prof_used += 2;
+  return e;
+}
+
+// One FP64 pass as digit passes: one transform per launch, so DST-Lambda-DST goes through the work vector
+// zb (free until the pass that writes z) and the fused sub-solve and product through z itself.
+template <int FLAGS>
+cudaError_t launch_digit_form(rfnse_ctx* c, const PassParams& p, int axis, int half, cudaStream_t s) {
+  cudaEvent_t stop;
+  cudaError_t e = prof_start<FLAGS>(c, s, &stop);
+  if (e != cudaSuccess) return e;
+  {
+    NvtxRange range("rfnse pass");
+    if constexpr ((FLAGS & F_LAM) != 0) {
+      PassParams q = p;
+      q.out = c->zb;
+      e = run_digit<F_DST | F_LAM>(c, q, axis, half, s);
+      q.in = c->zb;
+      q.out = p.out;
+      if (e == cudaSuccess) e = run_digit<F_DST>(c, q, axis, half, s);
+    } else if constexpr ((FLAGS & F_DSCALE) != 0) {
+      e = run_digit<F_DST | F_DSCALE>(c, p, axis, half, s);
+      if constexpr ((FLAGS & F_TOEP_X) != 0) {
+        PassParams q = p;
+        q.in = p.out;
+        if (e == cudaSuccess) e = run_digit<F_TOEP_X>(c, q, axis, half, s);
+      }
+    } else {
+      e = run_digit<FLAGS>(c, p, axis, half, s);
+    }
+  }
+  if (stop) {
+    cudaEventRecord(stop, s);
+    double fl, by;
+    pass_work<double, double2, double2, double2, double2, FLAGS>(p, fl, by);
+    c->prof_flops += fl;
+    c->prof_bytes += by;
+  }
+  cudaStreamCaptureStatus cap_st = cudaStreamCaptureStatusNone;
+  if (e == cudaSuccess && c->debug && cudaStreamIsCapturing(s, &cap_st) == cudaSuccess &&
+      cap_st == cudaStreamCaptureStatusNone) {
+    char what[96];
+    std::snprintf(what, sizeof what, "digit line pass (flags %d, axis stride %lld)", FLAGS, p.stride);
+    const void* outs[3] = {(FLAGS & (F_DST | F_DSCALE)) ? p.out : nullptr,
+                           (FLAGS & (F_TOEP_X | F_TOEP_ACC)) ? p.acc_out : nullptr,
+                           (FLAGS & F_INSCALE) ? (const void*)p.copy_out : nullptr};
+    const int elems[3] = {16, 16, 16};
+    if (p.gdyn) outs[0] = outs[2] = nullptr;  // device-resolved operands: not known on the host
+    return debug_after_pass(c, s, what, outs, elems, 3, c->N);
+  }
+  return e;
+}
+
+// One pass of the solver along `axis`: the digit form where it pays (or where the tuner found it fastest), the
+// line pass otherwise.  To the tuner the digit form is one more geometry (variant 2) of the configuration.
+template <typename R, typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
+cudaError_t solver_pass(rfnse_ctx* c, const PassParams& p, int axis, int half, cudaStream_t s) {
+  if constexpr (!digit_form<R, TIN, TOUT, TACCI, TACCO, FLAGS>()) {
+    return launch_pass<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s);
+  } else {
+    if (c->param_rec || !digit_possible(c, axis)) return launch_pass<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s);
+    auto launch = [c, p, axis, half, s](const PassGeom& g) {
+      return g.variant == 2 ? launch_digit_form<FLAGS>(c, p, axis, half, s)
+                            : launch_pass_geom<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s, g);
+    };
+    PassGeom g = default_pass_geometry<FLAGS>(p, false);
+    if (digit_pays(c, axis)) g = PassGeom{1, 1, 2};
+    if (c->tune_rec || !c->tune.empty()) {
+      const unsigned long long key = pass_key<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p);
+      if (c->tune_rec) {  // rfnse_autotune is recording the solver's pass configurations
+        bool seen = false;
+        for (const TuneRecord& r : *c->tune_rec) seen = seen || r.key == key;
+        if (!seen) {
+          TuneRecord r;
+          r.key = key;
+          r.dflt = g;
+          r.cands = pass_candidates<FLAGS>(p, false, sizeof(cv<R>));
+          r.cands.push_back(PassGeom{1, 1, 2});
+          r.launch = launch;
+          c->tune_rec->push_back(std::move(r));
+        }
+      } else {
+        const auto it = c->tune.find(key);
+        if (it != c->tune.end()) {
+          g = it->second;
+          c->tuned_launches += 1;
+        }
+      }
+    }
+    return launch(g);
+  }
+}
+
+}  // namespace rfnse

@@ -88,7 +88,8 @@ struct SolveCfg {
 };
 
 // Geometry of a line-pass launch (passes.cuh): lines per block, threads per line, kernel variant
-// (1 = the prefetching fixed-length FP32 kernel, 0 = k_line_pass).
+// (0 = k_line_pass, 1 = the prefetching fixed-length FP32 kernel, 2 = digit passes, digit.cuh: their
+// tiles are fixed, B and nt are not used).
 struct PassGeom {
   int B, nt, variant;
 };
@@ -290,6 +291,11 @@ struct rfnse_ctx {
   // (double-float, 8 B each); null when some axis has no fixed-length FFT
   void* twdf[3] = {nullptr, nullptr, nullptr};
   void* circdf[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
+  // digit passes (digit.cuh): per axis the digit tables of S and of mu_a T_0 (entry = integer * 2^exp; the
+  // first step's mu_a / 2 is one less in the exponent); null when the axis has none
+  void* digS[3] = {nullptr, nullptr, nullptr};
+  void* digT[3] = {nullptr, nullptr, nullptr};
+  int digT_exp[3] = {0, 0, 0};
   // mixed form: T u of each history vector, recovered from the final FP64 residual of the solve
   // that produced it (so the right-hand side two steps later needs no Toeplitz product)
   double2* Tu[3] = {nullptr, nullptr, nullptr};

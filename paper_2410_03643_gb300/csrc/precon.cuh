@@ -5,6 +5,7 @@
 #include <utility>
 #include "internal.cuh"
 #include "passes.cuh"
+#include "digit.cuh"
 
 namespace rfnse {
 
@@ -111,12 +112,12 @@ cudaError_t run_precon_pc(rfnse_ctx* c, const TIN* v, const double* in_scale, do
       p.acc_out = w;
       if (dot0) {
         with_dot0(p);
-        return launch_pass<R, TIN, TZ, double2, double2, IS | F_DSCALE | TX | (MATVEC ? F_DOT0 : 0)>(c, p, s);
+        return solver_pass<R, TIN, TZ, double2, double2, IS | F_DSCALE | TX | (MATVEC ? F_DOT0 : 0)>(c, p, 0, h, s);
       }
-      return launch_pass<R, TIN, TZ, double2, double2, IS | F_DSCALE | TX>(c, p, s);
+      return solver_pass<R, TIN, TZ, double2, double2, IS | F_DSCALE | TX>(c, p, 0, h, s);
     }
     p.acc_out = wtmp;
-    if ((e = launch_pass<R, TIN, TZ, double2, TW, IS | F_DSCALE | TX>(c, p, s)) != cudaSuccess) return e;
+    if ((e = solver_pass<R, TIN, TZ, double2, TW, IS | F_DSCALE | TX>(c, p, 0, h, s)) != cudaSuccess) return e;
   } else {
     if (c->d == 1) {
       PassParams p = base_params<R>(c, 0, h);
@@ -126,36 +127,36 @@ cudaError_t run_precon_pc(rfnse_ctx* c, const TIN* v, const double* in_scale, do
       with_dyn(p);
       if (dot0) {
         with_dot0(p);
-        return launch_pass<R, TIN, TZ, double2, double2,
-                           IS | F_DST | CF | F_LAM | F_DSCALE | TX | (MATVEC ? F_DOT0 : 0)>(c, p, s);
+        return solver_pass<R, TIN, TZ, double2, double2,
+                           IS | F_DST | CF | F_LAM | F_DSCALE | TX | (MATVEC ? F_DOT0 : 0)>(c, p, 0, h, s);
       }
-      return launch_pass<R, TIN, TZ, double2, double2, IS | F_DST | CF | F_LAM | F_DSCALE | TX>(c, p, s);
+      return solver_pass<R, TIN, TZ, double2, double2, IS | F_DST | CF | F_LAM | F_DSCALE | TX>(c, p, 0, h, s);
     }
     {  // first axis: forward DST (and the Arnoldi normalisation)
       PassParams p = base_params<R>(c, 0, h);
       p.in = v; p.in_scale = in_scale; p.copy_out = copy_v; p.out = t1;
       with_dyn(p);
       p.zbase = nullptr;
-      if ((e = launch_pass<R, TIN, TMP, double2, double2, IS | F_DST | CF>(c, p, s)) != cudaSuccess) return e;
+      if ((e = solver_pass<R, TIN, TMP, double2, double2, IS | F_DST | CF>(c, p, 0, h, s)) != cudaSuccess) return e;
     }
     TMP* cur = t1;
     TMP* nxt = t2;
     for (int a2 = 1; a2 < c->d - 1; ++a2) {  // middle axes (d = 3): forward DST
       PassParams p = base_params<R>(c, a2, h);
       p.in = cur; p.out = nxt; p.skip = dyn.skip;
-      if ((e = launch_pass<R, TMP, TMP, double2, double2, F_DST | CF>(c, p, s)) != cudaSuccess) return e;
+      if ((e = solver_pass<R, TMP, TMP, double2, double2, F_DST | CF>(c, p, a2, h, s)) != cudaSuccess) return e;
       std::swap(cur, nxt);
     }
     {  // last axis: DST, multiply by i s/(w + i Lambda), DST
       PassParams p = base_params<R>(c, c->d - 1, h);
       p.in = cur; p.out = nxt; p.lamfac = Tables<R>::lamfac(c, h); p.skip = dyn.skip;
-      if ((e = launch_pass<R, TMP, TMP, double2, double2, F_DST | CF | F_LAM>(c, p, s)) != cudaSuccess) return e;
+      if ((e = solver_pass<R, TMP, TMP, double2, double2, F_DST | CF | F_LAM>(c, p, c->d - 1, h, s)) != cudaSuccess) return e;
       std::swap(cur, nxt);
     }
     for (int a2 = c->d - 2; a2 >= 1; --a2) {  // middle axes: inverse DST (S is involutory)
       PassParams p = base_params<R>(c, a2, h);
       p.in = cur; p.out = nxt; p.skip = dyn.skip; p.inv_dft = 1;
-      if ((e = launch_pass<R, TMP, TMP, double2, double2, F_DST | CF>(c, p, s)) != cudaSuccess) return e;
+      if ((e = solver_pass<R, TMP, TMP, double2, double2, F_DST | CF>(c, p, a2, h, s)) != cudaSuccess) return e;
       std::swap(cur, nxt);
     }
     {  // first axis: inverse DST, (wI + D)^{-1} sub-solve, optional Toeplitz along x
@@ -164,7 +165,7 @@ cudaError_t run_precon_pc(rfnse_ctx* c, const TIN* v, const double* in_scale, do
       p.Dr = Tables<R>::Dr(c, D); p.dfac = Tables<R>::dfac(c);
       p.acc_in = w_add; p.acc_out = wtmp; p.ca = a; p.cb = b; p.inv_dft = 1;
       with_dyn(p);
-      if ((e = launch_pass<R, TMP, TZ, double2, TW, F_DST | CF | F_DSCALE | TX>(c, p, s)) != cudaSuccess) return e;
+      if ((e = solver_pass<R, TMP, TZ, double2, TW, F_DST | CF | F_DSCALE | TX>(c, p, 0, h, s)) != cudaSuccess) return e;
     }
   }
   if (MATVEC) {
@@ -177,13 +178,13 @@ cudaError_t run_precon_pc(rfnse_ctx* c, const TIN* v, const double* in_scale, do
         p.acc_out = w;
         if (dot0) {
           with_dot0(p);
-          e = launch_pass<R, TZ, TZ, TW, double2, F_TOEP_ACC | F_DOT0>(c, p, s);
+          e = solver_pass<R, TZ, TZ, TW, double2, F_TOEP_ACC | F_DOT0>(c, p, a2, h, s);
         } else {
-          e = launch_pass<R, TZ, TZ, TW, double2, F_TOEP_ACC>(c, p, s);
+          e = solver_pass<R, TZ, TZ, TW, double2, F_TOEP_ACC>(c, p, a2, h, s);
         }
       } else {
         p.acc_out = wtmp;
-        e = launch_pass<R, TZ, TZ, TW, TW, F_TOEP_ACC>(c, p, s);
+        e = solver_pass<R, TZ, TZ, TW, TW, F_TOEP_ACC>(c, p, a2, h, s);
       }
       if (e != cudaSuccess) return e;
     }

@@ -72,12 +72,12 @@ cudaError_t run_matvec_fp64(rfnse_ctx* c, const double2* z, const double* D, dou
   {
     PassParams p = base_params<double>(c, 0, h);
     p.in = z; p.Dr = D; p.acc_in = add; p.acc_out = w; p.ca = a; p.cb = b; p.skip = skip;
-    if ((e = launch_pass<double, double2, double2, double2, double2, F_TOEP_X>(c, p, s)) != cudaSuccess) return e;
+    if ((e = solver_pass<double, double2, double2, double2, double2, F_TOEP_X>(c, p, 0, h, s)) != cudaSuccess) return e;
   }
   for (int a2 = 1; a2 < c->d; ++a2) {
     PassParams p = base_params<double>(c, a2, h);
     p.in = z; p.acc_in = w; p.acc_out = w; p.cb = b; p.skip = skip;
-    if ((e = launch_pass<double, double2, double2, double2, double2, F_TOEP_ACC>(c, p, s)) != cudaSuccess) return e;
+    if ((e = solver_pass<double, double2, double2, double2, double2, F_TOEP_ACC>(c, p, a2, h, s)) != cudaSuccess) return e;
   }
   return cudaSuccess;
 }
@@ -90,13 +90,13 @@ cudaError_t run_dst(rfnse_ctx* c, int axis, const double2* in, double2* out, int
   }
   PassParams p = base_params<double>(c, axis, 0);
   p.in = in; p.out = out;
-  return launch_pass<double, double2, double2, double2, double2, F_DST>(c, p, c->stream);
+  return solver_pass<double, double2, double2, double2, double2, F_DST>(c, p, axis, 0, c->stream);
 }
 
 cudaError_t run_toeplitz(rfnse_ctx* c, int axis, const double2* in, double2* out, int half) {
   PassParams p = base_params<double>(c, axis, half ? 1 : 0);
   p.in = in; p.acc_in = nullptr; p.acc_out = out; p.cb = kOne;
-  return launch_pass<double, double2, double2, double2, double2, F_TOEP_ACC>(c, p, c->stream);
+  return solver_pass<double, double2, double2, double2, double2, F_TOEP_ACC>(c, p, axis, half ? 1 : 0, c->stream);
 }
 
 cudaError_t run_apply_prec(rfnse_ctx* c, const double2* v, double2* z, const double* D, int half, int precision) {
@@ -509,8 +509,11 @@ static rfnse_status solve_graph(rfnse_ctx* c, const double* D, const double2* f,
   {  // kernels the graph executed: 2 at the start, per Arnoldi step its passes and the MGS kernel,
      // per cycle the cycle start, back-substitution, update and residual kernels
     const int d = c->d;
-    const long long step_k = (d == 1 ? 1 : 3 * d - 2) + 1;
-    const long long cycle_k = mixed ? 1 + 1 + d + 1 + 1 : 1 + 1 + 1 + (d == 1 ? 1 : 2 * d - 1) + d + 1;
+    // a digit form makes two launches of the DST-Lambda-DST pass and of the fused x pass
+    const int lam_k = !mixed && c->p.precond == 0 && c->tune.empty() && digit_pays(c, d - 1) ? 1 : 0;
+    const int fused_k = !mixed && c->p.precond == 0 && c->tune.empty() && digit_pays(c, 0) ? 1 : 0;
+    const long long step_k = (d == 1 ? 1 : 3 * d - 2) + lam_k + fused_k + 1;
+    const long long cycle_k = mixed ? 1 + 1 + d + 1 + 1 : 1 + 1 + 1 + (d == 1 ? 1 : 2 * d - 1) + lam_k + d + 1;
     const long long cycles = mixed ? pk.outer : (pk.it > 0 ? pk.outer + 1 : 0);
     count_launch(2 + step_k * pk.it + cycle_k * cycles);
   }
