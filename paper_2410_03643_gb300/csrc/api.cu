@@ -135,10 +135,9 @@ void free_ctx(rfnse_ctx* c) {
   cudaFree(c->nrm_part);
   cudaFree(c->tape);
   cudaFree(c->adj_red);
+  cudaFree(c->dig_mem);
   for (int a = 0; a < 3; ++a) {
     cudaFree(c->twdf[a]);
-    cudaFree(c->digS[a]);
-    cudaFree(c->digT[a]);
     for (int h = 0; h < 2; ++h) cudaFree(c->circdf[h][a]);
   }
   for (int a = 0; a < 3; ++a) {
@@ -290,14 +289,34 @@ int rfnse_create(const rfnse_params* p, void* stream, rfnse_ctx** out) {
       }
     }
   }
-  if (c->d > 1)  // digit passes of the axes that have them
-    for (int a = 0; a < c->d; ++a) {
-      DigitShape sh;
-      if (!digit_shape(c->n[a], &sh)) continue;
-      chk(dev_alloc(&c->digS[a], digit_table_bytes(sh)));
-      chk(dev_alloc(&c->digT[a], digit_table_bytes(sh)));
-      c->digT_exp[a] = digit_exp_toeplitz(p->alpha, c->mu[a]);
+  if (digit_context(c)) {  // the digit tables of every axis that has them, one allocation
+    size_t off = 0;
+    for (int pass = 0; pass < 2; ++pass) {
+      off = 0;
+      for (int a = 0; a < c->d; ++a) {
+        DigitShape sh;
+        if (!digit_shape(c->n[a], &sh)) continue;
+        const size_t bytes = digit_table_bytes(sh);
+        const size_t bytes32 = p->precision == 1 && p->precond == 0 && sh.kb == 1 ? digit_table_bytes(sh, kDigits32) : 0;
+        if (pass == 1) {
+          char* m = static_cast<char*>(c->dig_mem) + off;
+          c->digS[a] = m;
+          c->digT[a] = m + bytes;
+          c->digT_exp[a] = digit_exp_toeplitz(p->alpha, c->mu[a]);
+          if (bytes32) {
+            c->digS32[a] = m + 2 * bytes;
+            c->digT32[a] = m + 2 * bytes + bytes32;
+          }
+        }
+        off += 2 * (bytes + bytes32);
+      }
+      if (off == 0) break;
+      if (pass == 0) {
+        chk(dev_alloc(&c->dig_mem, off));
+        if (e != cudaSuccess) break;
+      }
     }
+  }
   c->red_blocks = choose_reduce_blocks(N);
   {
     const char* dbg = std::getenv("RFNSE_DEBUG");
@@ -332,8 +351,13 @@ int rfnse_create(const rfnse_params* p, void* stream, rfnse_ctx** out) {
   for (int a = 0; a < c->d; ++a) {
     launch_setup_axis(c->c, c->n[a], c->L[a], c->lam[a], c->circ[a], c->tw64[a], c->tw32[a], c->stream);
     if (c->digS[a]) {
-      launch_setup_digits(c->c, c->n[a], 1.0, 0, digit_exp_dst(c->n[a]), a == 0, c->digS[a], c->stream);
-      launch_setup_digits(c->c, c->n[a], c->mu[a], 1, c->digT_exp[a], a == 0, c->digT[a], c->stream);
+      const int es = digit_exp_dst(c->n[a]), et = c->digT_exp[a];
+      launch_setup_digits(c->c, c->n[a], 1.0, 0, es, a == 0, kDigits, c->digS[a], c->stream);
+      launch_setup_digits(c->c, c->n[a], c->mu[a], 1, et, a == 0, kDigits, c->digT[a], c->stream);
+      if (c->digS32[a]) {
+        launch_setup_digits(c->c, c->n[a], 1.0, 0, es, a == 0, kDigits32, c->digS32[a], c->stream);
+        launch_setup_digits(c->c, c->n[a], c->mu[a], 1, et, a == 0, kDigits32, c->digT32[a], c->stream);
+      }
     }
     if (p->precond == 1)
       launch_setup_circ(c->c, c->n[a], c->L[a], c->lamC[a], c->chirp64[a], c->chirp32[a], c->bspec64[a],

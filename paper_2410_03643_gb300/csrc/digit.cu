@@ -31,16 +31,18 @@ constexpr int kRowPitch = kDigLines * 16 + 16;  // staged results: a row's 16 li
 template <int KB> constexpr int digit_bytes() { return (16 * KB * kLbo + 127) & ~127; }
 template <int KB> constexpr int digit_smem() { return kCtrl + digit_bytes<KB>() + kDigStages * kDigChunkBytes; }
 
-// x as a fixed-point integer on the scale of exponent emax: |X| < 2^61, x = X 2^(emax - 1083)
-__device__ __forceinline__ long long to_fixed(double x, int emax) {
-  const int hi = __double2hiint(x);
-  const unsigned lo = (unsigned)__double2loint(x);
-  const int e = (hi >> 20) & 0x7ff;
-  const unsigned mh = ((unsigned)hi & 0xfffffu) | (e ? 0x100000u : 0u);
-  const int sh = emax - (e ? e : 1);
-  unsigned long long m = (((unsigned long long)mh << 32) | lo) << 8;
-  m = sh > 63 ? 0ull : m >> sh;
-  return hi < 0 ? -(long long)m : (long long)m;
+// x as a fixed-point integer on the scale of exponent emax: |X| < 2^61, x = X 2^(emax - 1083), by 32-bit
+// shifts (what lies below 2^-61 of the scale is cut off).  All integer: an FP64 operation takes half a cycle of
+// an SM, an integer one 1/64.
+__device__ __forceinline__ long long to_fixed(uint32_t hi, uint32_t lo, int emax) {
+  const int e = (int)((hi >> 20) & 0x7ff);
+  const uint32_t mh = (hi & 0xfffffu) | (e ? 0x100000u : 0u);
+  const int sh = emax - max(e, 1);
+  const uint32_t H = __funnelshift_l(lo, mh, 8), L = lo << 8;
+  const uint32_t l = __funnelshift_rc(__funnelshift_rc(L, H, sh), 0u, max(sh - 32, 0));
+  const uint32_t u = __funnelshift_rc(H, 0u, sh);
+  const long long X = (long long)(((unsigned long long)u << 32) | l);
+  return (int)hi < 0 ? -X : X;
 }
 
 // v 2^ex rounded to nearest (truncated below the normal range, infinity above it)
@@ -161,6 +163,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
 
   double va[8];
   [[maybe_unused]] double vb[8];
+  const bool mid = FOLD && 2 * slot_pos(7) == n - 1;  // the thread's last entry is the middle of the line
   {
     const double2* in = reinterpret_cast<const double2*>(p.in);
     double2* cpy = p.copy_out;
@@ -174,39 +177,42 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
         sc = *p.in_scale;
       }
     }
+    if constexpr (FOLD) {
+      const bool ok = line0 + l < nline;
+      const long long g0 = base0 + (line0 + l) * lstep, g1 = g0 + (long long)(n - 1 - slot_pos(0)) * estep;
+      const long long step = (xax ? 16 : 1) * estep;
+      const long long g = g0 + slot_pos(0) * estep;
+      const double* s = reinterpret_cast<const double*>(in + g) + part;
+      const double* t = reinterpret_cast<const double*>(in + g1) + part;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      const int q = slot_pos(i);
-      va[i] = 0.0;
-      if constexpr (FOLD) {
-        vb[i] = 0.0;
-        if (line0 + l < nline) {
-          const double* s = reinterpret_cast<const double*>(in + base0 + (line0 + l) * lstep) + part;
-          va[i] = s[2 * (q * estep)];
-          if (2 * q != n - 1) vb[i] = s[2 * ((n - 1 - q) * estep)];
-        }
-      } else {
-        const int sl = q >> a.log2N, pos = q - (sl << a.log2N);
-        const long long ln = line0 + sl * kDigLines + l;
-        if (ln < nline && pos < n) va[i] = reinterpret_cast<const double*>(in + base0 + ln * lstep + pos * estep)[part];
+      for (int i = 0; i < 8; ++i) {
+        va[i] = ok ? s[2 * i * step] : 0.0;
+        vb[i] = ok && !(i == 7 && mid) ? t[-2 * i * step] : 0.0;
       }
-    }
-    if constexpr ((FLAGS & F_INSCALE) != 0) {
+      if constexpr ((FLAGS & F_INSCALE) != 0) {
+        double* d = reinterpret_cast<double*>(cpy + g) + part;
+        double* f = reinterpret_cast<double*>(cpy + g1) + part;
+        const bool wr = ok && h == 0 && mb == 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          va[i] *= sc;
+          vb[i] *= sc;
+          if (wr) d[2 * i * step] = va[i];
+          if (wr && !(i == 7 && mid)) f[-2 * i * step] = vb[i];
+        }
+      }
+    } else {
 #pragma unroll
       for (int i = 0; i < 8; ++i) {
         const int q = slot_pos(i);
-        va[i] *= sc;
-        if constexpr (FOLD) {
-          vb[i] *= sc;
-          if (h == 0 && mb == 0 && line0 + l < nline) {
-            double* d = reinterpret_cast<double*>(cpy + base0 + (line0 + l) * lstep) + part;
-            d[2 * (q * estep)] = va[i];
-            if (2 * q != n - 1) d[2 * ((n - 1 - q) * estep)] = vb[i];
-          }
-        } else {
-          const int sl = q >> a.log2N, pos = q - (sl << a.log2N);
-          const long long ln = line0 + sl * kDigLines + l;
-          if (ln < nline && pos < n) reinterpret_cast<double*>(cpy + base0 + ln * lstep + pos * estep)[part] = va[i];
+        const int sl = q >> a.log2N, pos = q - (sl << a.log2N);
+        const long long ln = line0 + sl * kDigLines + l;
+        const long long g = base0 + ln * lstep + pos * estep;
+        const bool ok = ln < nline && pos < n;
+        va[i] = ok ? reinterpret_cast<const double*>(in + g)[part] : 0.0;
+        if constexpr ((FLAGS & F_INSCALE) != 0) {
+          va[i] *= sc;
+          if (ok) reinterpret_cast<double*>(cpy + g)[part] = va[i];
         }
       }
     }
@@ -237,11 +243,11 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       long long y[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
-        y[k] = to_fixed(va[i + k], emax);
-        if constexpr (FOLD) {
-          const long long m = to_fixed(vb[i + k], emax);
-          if (h == 0) y[k] += m;
-          else y[k] = 2 * slot_pos(i + k) != n - 1 ? y[k] - m : 0;
+        y[k] = to_fixed((uint32_t)__double2hiint(va[i + k]), (uint32_t)__double2loint(va[i + k]), emax);
+        if constexpr (FOLD) {  // + or - the mirror image; the middle belongs to the sums alone
+          y[k] += to_fixed((uint32_t)__double2hiint(vb[i + k]) ^ ((uint32_t)h << 31),
+                           (uint32_t)__double2loint(vb[i + k]), emax);
+          if (i + k == 7 && h == 1 && mid) y[k] = 0;
         }
       }
       uint32_t d[kDigits];
@@ -302,9 +308,9 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
     }
   }
   __syncwarp();
-  if (!tc::mbar_wait(b_done, 0)) *s_fail = 1;
+  if (uwarp == 0 && !tc::mbar_wait(b_done, 0) && lane == 0) *s_fail = 1;
+  __syncthreads();  // the other warps sleep here rather than poll
   tc::fence_after();
-  __syncthreads();
   if (*s_fail) {  // uniform: a wait gave up; wait for the copies in flight, free TMEM and leave
     if (tid == 32) {
       for (int c = issued - kDigStages; c < issued; ++c)
@@ -426,14 +432,13 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
   };
   if constexpr (PAIR) {  // y_j = e_j + o_j, y_{N-j} = e_j - o_j; this block finishes eight of the lines
     constexpr int ITEMS = 128 * 8 / NT;
-#pragma unroll 2
+    int r = xax ? (tid & 127) : (tid >> 3), ln = 8 * h + (xax ? (tid >> 7) : (tid & 7));
+    long long g = base0 + (line0 + ln) * lstep + (mb * 128 + r) * estep;
+    long long g2 = base0 + (line0 + ln) * lstep + (n - 1 - mb * 128 - r) * estep;
+    const long long dg = xax ? (NT / 128) * lstep : (NT / 8) * estep;
+#pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-      const int e = it * NT + tid;
-      const int r = xax ? (e & 127) : (e >> 3), ln = 8 * h + (xax ? (e >> 7) : (e & 7));
-      const int q = mb * 128 + r;
-      const bool ok = line0 + ln < nline, two = 2 * q != n - 1;
-      const long long g = base0 + (line0 + ln) * lstep + q * estep;
-      const long long g2 = base0 + (line0 + ln) * lstep + (n - 1 - q) * estep;
+      const bool ok = line0 + ln < nline, two = 2 * (mb * 128 + r) != n - 1;
       const Operands o1 = fetch(g, ok), o2 = fetch(g2, ok && two);
       const uint32_t at = sdig + r * kRowPitch + ln * 16;
       long long er, ei, dr, di;
@@ -441,28 +446,34 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       tc::ld_cluster(at, 1, dr, di);
       if (ok) emit(g, er + dr, ei + di, ln, o1);
       if (ok && two) emit(g2, er - dr, ei - di, ln, o2);
+      g += dg;
+      g2 += xax ? dg : -dg;
+      if (xax) ln += NT / 128;
+      else r += NT / 8;
     }
     tc::cluster_sync();
   } else {
     constexpr int ITEMS = 128 * kDigLines / NT;
-#pragma unroll 2
+    int r = xax ? (tid & 127) : (tid >> 4), ln = xax ? (tid >> 7) : (tid & 15);
+    long long g = base0 + (line0 + ln) * lstep + (long long)(2 * (mb * 128 + r) + h) * estep;  // FOLD
+    const long long dg = xax ? (NT / 128) * lstep : 2 * (NT / 16) * estep;
+#pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-      const int e = it * NT + tid;
-      const int r = xax ? (e & 127) : (e >> 4), ln = xax ? (e >> 7) : (e & 15);
-      int pos;
+      int pos = 2 * (mb * 128 + r) + h;
       long long line = line0 + ln;
-      if constexpr (FOLD) {
-        pos = 2 * (mb * 128 + r) + h;
-      } else {
+      if constexpr (!FOLD) {
         const int sl = r >> a.log2N;
         pos = r - (sl << a.log2N);
         line += sl * kDigLines;
+        g = base0 + line * lstep + pos * estep;
       }
       const bool ok = line < nline && pos < n;
-      const long long g = base0 + line * lstep + pos * estep;
       const Operands o = fetch(g, ok);
       const longlong2 v = *reinterpret_cast<const longlong2*>(dig + r * kRowPitch + ln * 16);
       if (ok) emit(g, v.x, v.y, ln, o);
+      g += dg;
+      if (xax) ln += NT / 128;
+      else r += NT / 16;
     }
   }
   if constexpr ((FLAGS & F_DOT0) != 0) block_sum_store(dot, p.dot_part + blockIdx.x);
@@ -509,8 +520,11 @@ bool digit_possible(const rfnse_ctx* c, int axis) { return c->digS[axis] != null
 // A single tile takes 8 us whatever its size, and a fused FFT pass is two launches here: below 8192 points
 // the FFT passes are as fast or faster (63 x 31: 15.4 / 24.0 us for S / T along x against 14.5 / 16.0 here,
 // but 15.4 against 29 for the fused pair), from 127^2 on these are (127^2: S 17.8 and 23.5 us along x and y
-// against 15; 511^2: 47 against 24, T 87 against 27; 255^3: S 2000 against 415, T 3870 against 475).
-bool digit_pays(const rfnse_ctx* c, int axis) { return c->N >= 8192 && digit_possible(c, axis); }
+// against 15; 511^2: 47 against 24, T 87 against 27; 255^3: S 2000 against 415, T 3870 against 475).  The
+// mixed form's residual products have double-float passes to beat: 255^3 860-970 against 480 us, but 511^2 33
+// against 27, and a batch of 16 grids of 127..511 points per axis took 24.9 ms with those and 25.9 with these
+// (a block here fills half an SM, so the instances' streams overlap less), hence from 2^20 points on.
+bool digit_context(const rfnse_ctx* c) { return c->d > 1 && c->N >= (c->p.precision == 1 ? 1 << 20 : 8192); }
 
 template <int FLAGS>
 cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s) {

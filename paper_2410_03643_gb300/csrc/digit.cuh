@@ -33,6 +33,8 @@ constexpr int kDigits = 7;        // digits of an entry = accumulators (weights)
 // result = sum_d D_d 2^(shift - 9d) in 64 bits: |D_0| < 2^17 for the Toeplitz rows (sum |c_k| = 2 c_0), and
 // < 2^23 for the sine rows of two 128-entry blocks
 constexpr int kDigShiftT = 45, kDigShiftS = 40;
+constexpr int kDigits32 = 3;      // of the FP32 passes (digit32.cu)
+constexpr int kDigExpBits = 61;   // operator entry = integer * 2^exp, |integer| <= 2^61
 constexpr int kDigCols = 32;      // columns of a tile: 16 lines, real and imaginary part
 constexpr int kDigLines = 16;
 constexpr int kDigChunkK = 32;    // operator entries along K per chunk: 128 rows x 32 x 2 B = 8 KB
@@ -52,32 +54,52 @@ inline bool digit_shape(int n, DigitShape* s) {
   return true;
 }
 // bytes of an operator's digit table: halves x row blocks x digits x K/32 chunks
-inline size_t digit_table_bytes(const DigitShape& s) {
-  return (size_t)s.halves * s.kb * kDigits * (s.kb * 128 / kDigChunkK) * kDigChunkBytes;
+inline size_t digit_table_bytes(const DigitShape& s, int digits = kDigits) {
+  return (size_t)s.halves * s.kb * digits * (s.kb * 128 / kDigChunkK) * kDigChunkBytes;
 }
 
 // The operator tables of one axis (set-up): S and mu_a T_0, each value = integer * 2^exp.
 // entry = 0: the DST-I, 1: the Toeplitz operator (coefficients c scaled by mu)
-void launch_setup_digits(const double* c, int n, double mu, int toeplitz, int exp, bool xax, void* table,
+// digits = kDigits: the FP64 passes' table; kDigits32: the FP32 passes'
+void launch_setup_digits(const double* c, int n, double mu, int toeplitz, int exp, bool xax, int digits, void* table,
                          cudaStream_t s);
 // exponent e with every |entry| <= 2^(e + 61)
 int digit_exp_dst(int n);
 int digit_exp_toeplitz(double alpha, double mu);
 
-// Whether the FP64 passes of an axis run as digit passes by default, whether they can, and one digit pass:
-// all storage FP64, FLAGS as for the line passes with one transform ([F_INSCALE |] F_DST, F_DST | F_LAM =
+// Whether a context has digit tables at all, whether the FP64 passes of an axis run as digit passes (by default;
+// the tuner may choose the line pass), and one digit pass: all storage FP64, FLAGS as for the line passes with one transform ([F_INSCALE |] F_DST, F_DST | F_LAM =
 // S x / (omega + i Lambda), F_DST | F_DSCALE, F_TOEP_X, F_TOEP_ACC [| F_DOT0]); half: the first step's mu_a / 2.
-bool digit_pays(const rfnse_ctx* c, int axis);
+bool digit_context(const rfnse_ctx* c);
 bool digit_possible(const rfnse_ctx* c, int axis);
 template <int FLAGS>
 cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s);
 
-// The passes that have a digit form: FP64 throughout, a sine transform or a Toeplitz product, and not the
-// fused pass of 1-D grids (one launch there, three as digit passes).
+// The FP32 passes of the mixed form: whether an axis has them, and one pass with the given storage types.
+bool digit32_possible(const rfnse_ctx* c, int axis);
+template <typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
+cudaError_t run_digit32(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s);
+
+// The passes that have a digit form: a sine transform or a Toeplitz product, and not the fused pass of 1-D
+// grids (one launch there, three as digit passes); FP64 throughout, or FP32 with the storage types of the
+// mixed form's Arnoldi step.
 template <typename R, typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
 constexpr bool digit_form() {
-  return sizeof(R) == 8 && sizeof(TIN) == 16 && sizeof(TOUT) == 16 && sizeof(TACCI) == 16 && sizeof(TACCO) == 16 &&
-         !(FLAGS & F_CIRC) && ((FLAGS & F_DST) || !(FLAGS & F_DSCALE)) && !((FLAGS & F_LAM) && (FLAGS & F_DSCALE));
+  if ((FLAGS & F_CIRC) || (!(FLAGS & F_DST) && (FLAGS & F_DSCALE)) || ((FLAGS & F_LAM) && (FLAGS & F_DSCALE)))
+    return false;
+  constexpr bool in16 = sizeof(TIN) == 16, out16 = sizeof(TOUT) == 16, ai16 = sizeof(TACCI) == 16,
+                 ao16 = sizeof(TACCO) == 16;
+  if (sizeof(R) == 8) return in16 && out16 && ai16 && ao16;
+  if (out16 || in16 != ((FLAGS & F_INSCALE) != 0)) return false;
+  if (FLAGS & F_DSCALE) return (FLAGS & F_TOEP_X) && !(FLAGS & F_DOT0) && ai16 && !ao16;
+  if (FLAGS & F_DST) return ai16 && ao16;
+  return (FLAGS & F_TOEP_ACC) && !ai16 && (ao16 || !(FLAGS & F_DOT0));
+}
+
+template <typename R, typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
+cudaError_t run_digit_any(rfnse_ctx* c, const PassParams& p, int axis, int half, cudaStream_t s) {
+  if constexpr (sizeof(R) == 8) return run_digit<FLAGS>(c, p, axis, half, s);
+  else return run_digit32<TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, axis, half, s);
 }
 
 // CUDA events around the launches of a profiled pass (rfnse_profile): the stop event, null when the pass
@@ -98,37 +120,40 @@ cudaError_t prof_start(rfnse_ctx* c, cudaStream_t s, cudaEvent_t* stop) {
   return e;
 }
 
-// One FP64 pass as digit passes: one transform per launch, so DST-Lambda-DST goes through the work vector
-// zb (free until the pass that writes z) and the fused sub-solve and product through z itself.
-template <int FLAGS>
+// One pass as digit passes: one transform per launch, so DST-Lambda-DST goes through the work vector zb
+// (free until the pass that writes z) and the fused sub-solve and product through z itself.
+// KIND: the kernel class under which rfnse_profile times it.
+template <typename R, typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS,
+          int KIND = FLAGS | (sizeof(R) == 4 ? 256 : 0)>
 cudaError_t launch_digit_form(rfnse_ctx* c, const PassParams& p, int axis, int half, cudaStream_t s) {
   cudaEvent_t stop;
-  cudaError_t e = prof_start<FLAGS>(c, s, &stop);
+  cudaError_t e = prof_start<KIND>(c, s, &stop);
   if (e != cudaSuccess) return e;
   {
     NvtxRange range("rfnse pass");
     if constexpr ((FLAGS & F_LAM) != 0) {
       PassParams q = p;
       q.out = c->zb;
-      e = run_digit<F_DST | F_LAM>(c, q, axis, half, s);
+      e = run_digit_any<R, TIN, TOUT, TACCI, TACCO, F_DST | F_LAM>(c, q, axis, half, s);
       q.in = c->zb;
       q.out = p.out;
-      if (e == cudaSuccess) e = run_digit<F_DST>(c, q, axis, half, s);
+      if (e == cudaSuccess) e = run_digit_any<R, TOUT, TOUT, TACCI, TACCO, F_DST>(c, q, axis, half, s);
     } else if constexpr ((FLAGS & F_DSCALE) != 0) {
-      e = run_digit<F_DST | F_DSCALE>(c, p, axis, half, s);
+      e = run_digit_any<R, TIN, TOUT, TACCI, TACCO, F_DST | F_DSCALE>(c, p, axis, half, s);
       if constexpr ((FLAGS & F_TOEP_X) != 0) {
         PassParams q = p;
         q.in = p.out;
-        if (e == cudaSuccess) e = run_digit<F_TOEP_X>(c, q, axis, half, s);
+        q.in_dyn_z = (p.gdyn && p.zbase) ? 1 : 0;
+        if (e == cudaSuccess) e = run_digit_any<R, TOUT, TOUT, TACCI, TACCO, F_TOEP_X>(c, q, axis, half, s);
       }
     } else {
-      e = run_digit<FLAGS>(c, p, axis, half, s);
+      e = run_digit_any<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, axis, half, s);
     }
   }
   if (stop) {
     cudaEventRecord(stop, s);
     double fl, by;
-    pass_work<double, double2, double2, double2, double2, FLAGS>(p, fl, by);
+    pass_work<R, TIN, TOUT, TACCI, TACCO, FLAGS>(p, fl, by);
     c->prof_flops += fl;
     c->prof_bytes += by;
   }
@@ -136,11 +161,12 @@ cudaError_t launch_digit_form(rfnse_ctx* c, const PassParams& p, int axis, int h
   if (e == cudaSuccess && c->debug && cudaStreamIsCapturing(s, &cap_st) == cudaSuccess &&
       cap_st == cudaStreamCaptureStatusNone) {
     char what[96];
-    std::snprintf(what, sizeof what, "digit line pass (flags %d, axis stride %lld)", FLAGS, p.stride);
+    std::snprintf(what, sizeof what, "digit line pass (flags %d, %s, axis stride %lld)", FLAGS,
+                  sizeof(R) == 4 ? "FP32" : "FP64", p.stride);
     const void* outs[3] = {(FLAGS & (F_DST | F_DSCALE)) ? p.out : nullptr,
                            (FLAGS & (F_TOEP_X | F_TOEP_ACC)) ? p.acc_out : nullptr,
                            (FLAGS & F_INSCALE) ? (const void*)p.copy_out : nullptr};
-    const int elems[3] = {16, 16, 16};
+    const int elems[3] = {(int)sizeof(TOUT), (int)sizeof(TACCO), 16};
     if (p.gdyn) outs[0] = outs[2] = nullptr;  // device-resolved operands: not known on the host
     return debug_after_pass(c, s, what, outs, elems, 3, c->N);
   }
@@ -154,13 +180,13 @@ cudaError_t solver_pass(rfnse_ctx* c, const PassParams& p, int axis, int half, c
   if constexpr (!digit_form<R, TIN, TOUT, TACCI, TACCO, FLAGS>()) {
     return launch_pass<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s);
   } else {
-    if (c->param_rec || !digit_possible(c, axis)) return launch_pass<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s);
+    const bool possible = sizeof(R) == 8 ? digit_possible(c, axis) : digit32_possible(c, axis);
+    if (c->param_rec || !possible) return launch_pass<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s);
     auto launch = [c, p, axis, half, s](const PassGeom& g) {
-      return g.variant == 2 ? launch_digit_form<FLAGS>(c, p, axis, half, s)
+      return g.variant == 2 ? launch_digit_form<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, axis, half, s)
                             : launch_pass_geom<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s, g);
     };
-    PassGeom g = default_pass_geometry<FLAGS>(p, false);
-    if (digit_pays(c, axis)) g = PassGeom{1, 1, 2};
+    PassGeom g{1, 1, 2};
     if (c->tune_rec || !c->tune.empty()) {
       const unsigned long long key = pass_key<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p);
       if (c->tune_rec) {  // rfnse_autotune is recording the solver's pass configurations
@@ -170,8 +196,7 @@ cudaError_t solver_pass(rfnse_ctx* c, const PassParams& p, int axis, int half, c
           TuneRecord r;
           r.key = key;
           r.dflt = g;
-          r.cands = pass_candidates<FLAGS>(p, false, sizeof(cv<R>));
-          r.cands.push_back(PassGeom{1, 1, 2});
+          r.cands = pass_candidates<FLAGS>(p, sizeof(R) == 4 && fixed_fft_length(p.log2L), sizeof(cv<R>));
           r.launch = launch;
           c->tune_rec->push_back(std::move(r));
         }

@@ -17,7 +17,7 @@ __host__ __device__ inline int digit_slot_pos(int kap, bool xax) {
 }
 
 __global__ void k_digit_table(const double* __restrict__ c, int n, double mu, int toeplitz, int exp, int xax,
-                              int kb, int halves, __half* __restrict__ table) {
+                              int kb, int halves, int digits, __half* __restrict__ table) {
   const int K = 128 * kb, N = n + 1;
   const long long total = (long long)halves * K * K;
   for (long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x; t < total;
@@ -59,31 +59,44 @@ __global__ void k_digit_table(const double* __restrict__ c, int n, double mu, in
       }
     }
     const double a = f * g, ae = fma(f, g, -a) + f * e + fe * g;
+    const int nk = K / kDigChunkK;
+    const int chunk = kap / kDigChunkK, kin = kap % kDigChunkK, mb = row >> 7, r = row & 127;
+    // K-major core matrices: 8 rows x 8 entries, rows of 16 B; 16 row groups, then the next 8 entries
+    const size_t off = (size_t)(kin >> 3) * 1024 + (size_t)(r >> 3) * 64 + (size_t)(r & 7) * 8 + (kin & 7);
+    auto put = [&](int i, __half d) {
+      const size_t ch = (((size_t)h * kb + mb) * digits + i) * nk + chunk;
+      table[ch * (kDigChunkBytes / 2) + off] = d;
+    };
+    if (digits == kDigits32) {  // nearest integer (at most 256), then FP16 remainders, row by row
+      auto put32 = [&](int i, __half d) { table[(((size_t)h * digits + i) * 128 + row) * 128 + kap] = d; };
+      const double s = ldexp(a, 8 - kDigExpBits - exp);
+      const double d0 = rint(s), r1 = (s - d0) * 2048.0;
+      const __half d1 = __double2half(r1);
+      put32(0, __double2half(d0));
+      put32(1, d1);
+      put32(2, __double2half((r1 - (double)__half2float(d1)) * 2048.0));
+      continue;
+    }
     long long v = llrint(ldexp(a, -exp)) + llrint(ldexp(ae, -exp));
     long long bias = 0;
     for (int i = 0; i < kDigits; ++i) bias += 256LL << (9 * i);
     v += bias;
-    const int nk = K / kDigChunkK;
-    const int chunk = kap / kDigChunkK, kin = kap % kDigChunkK, mb = row >> 7, r = row & 127;
     for (int i = 0; i < kDigits; ++i) {
       const long long u = v >> (9 * (kDigits - 1 - i));
       const int dg = (int)(i == 0 ? u : (u & 511)) - 256;
-      const size_t ch = (((size_t)h * kb + mb) * kDigits + i) * nk + chunk;
-      // K-major core matrices: 8 rows x 8 entries, rows of 16 B; 16 row groups, then the next 8 entries
-      const size_t off = (size_t)(kin >> 3) * 1024 + (size_t)(r >> 3) * 64 + (size_t)(r & 7) * 8 + (kin & 7);
-      table[ch * (kDigChunkBytes / 2) + off] = __int2half_rn(dg);
+      put(i, __int2half_rn(dg));
     }
   }
 }
 
-void launch_setup_digits(const double* c, int n, double mu, int toeplitz, int exp, bool xax, void* table,
+void launch_setup_digits(const double* c, int n, double mu, int toeplitz, int exp, bool xax, int digits, void* table,
                          cudaStream_t s) {
   DigitShape sh;
   if (!digit_shape(n, &sh)) return;
   const long long total = (long long)sh.halves * 128 * sh.kb * 128 * sh.kb;
   count_launch();
   k_digit_table<<<(unsigned)((total + 127) / 128), 128, 0, s>>>(c, n, mu, toeplitz, exp, xax ? 1 : 0, sh.kb,
-                                                               sh.halves, reinterpret_cast<__half*>(table));
+                                                               sh.halves, digits, reinterpret_cast<__half*>(table));
 }
 
 // |entry| <= sqrt(2/N), N a power of two: sqrt(2/N) <= 2^ceil((1 - log2 N)/2)
@@ -91,7 +104,7 @@ int digit_exp_dst(int n) {
   int l = 0;
   while ((1 << l) < n + 1) ++l;
   const int e = -((l - 1) / 2);  // ceil((1 - l) / 2)
-  return e - 61;
+  return e - kDigExpBits;
 }
 
 // |entry| <= mu c_0, c_0 = Gamma(alpha + 1) / Gamma(alpha/2 + 1)^2 (every |c_k| <= c_0)
@@ -99,7 +112,7 @@ int digit_exp_toeplitz(double alpha, double mu) {
   const double g = std::tgamma(alpha / 2 + 1);
   int e = 0;
   std::frexp(mu * std::tgamma(alpha + 1) / (g * g) * (1.0 + 1e-9), &e);
-  return e - 61;
+  return e - kDigExpBits;
 }
 
 }  // namespace rfnse

@@ -293,9 +293,12 @@ struct rfnse_ctx {
   void* circdf[2][3] = {{nullptr, nullptr, nullptr}, {nullptr, nullptr, nullptr}};
   // digit passes (digit.cuh): per axis the digit tables of S and of mu_a T_0 (entry = integer * 2^exp; the
   // first step's mu_a / 2 is one less in the exponent); null when the axis has none
+  void* dig_mem = nullptr;  // the allocation behind these tables
   void* digS[3] = {nullptr, nullptr, nullptr};
   void* digT[3] = {nullptr, nullptr, nullptr};
   int digT_exp[3] = {0, 0, 0};
+  void* digS32[3] = {nullptr, nullptr, nullptr};  // the same for the FP32 passes of the mixed form
+  void* digT32[3] = {nullptr, nullptr, nullptr};
   // mixed form: T u of each history vector, recovered from the final FP64 residual of the solve
   // that produced it (so the right-hand side two steps later needs no Toeplitz product)
   double2* Tu[3] = {nullptr, nullptr, nullptr};

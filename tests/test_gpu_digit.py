@@ -82,3 +82,27 @@ def test_digit_passes_at_the_ends_of_the_number_range():
     # subnormal results are truncated to a multiple of 2^-1074, and their inputs are
     assert np.max(np.abs(y[1].real - (x[1].real.astype(np.longdouble) @ S).astype(float))) < 20 * 5e-324
     s.close()
+
+
+@pytest.mark.parametrize("n", [(255, 63, 127), (127, 255, 63), (31, 255, 255)])
+def test_fp32_digit_passes_in_the_mixed_form(n):
+    """Grids of 2^20 points and more: the FP32 preconditioner against the FP64 one (three FP32 roundings per
+    pass, 7 passes: 1e-6 is five times their sum), and two mixed steps against the FP64 form (both solved to
+    1e-10, so 1e-8 as everywhere for the mixed form)."""
+    from paper_2410_03643_gb300 import Solver
+    p = W.Problem(d=3, n=n, lo=(-6.0,) * 3, hi=(6.0,) * 3, alpha=1.6, rho=1.0, dt=0.01, tol=1e-10)
+    assert p.size >= 1 << 20
+    u0 = torch.from_numpy(W.u0_gaussian(p).reshape(-1).copy()).cuda()
+    m, f = Solver(p, precision=1), Solver(p, precision=0)
+    D = (p.rho * p.dt * u0.abs() ** 2).contiguous()
+    v = torch.from_numpy(W.random_field(p.shape, 5).reshape(-1).copy()).cuda()
+    a, b = m.apply_prec(v, D, precision=1), f.apply_prec(v, D)
+    assert float((a - b).norm() / b.norm()) < 1e-6
+    out = []
+    for s in (m, f):
+        s.set_state(u0)
+        its, _ = s.run(2)
+        out.append((s.get_state()[1], its))
+        s.close()
+    assert float((out[0][0] - out[1][0]).norm() / out[1][0].norm()) < 1e-8
+    assert np.all(np.abs(out[0][1].astype(int) - out[1][1].astype(int)) <= 4)
