@@ -517,14 +517,14 @@ cudaError_t launch_digit(const PassParams& p, const DigitArgs& a, unsigned grid,
 
 bool digit_possible(const rfnse_ctx* c, int axis) { return c->digS[axis] != nullptr; }
 
-// A single tile takes 8 us whatever its size, and a fused FFT pass is two launches here: below 8192 points
-// the FFT passes are as fast or faster (63 x 31: 15.4 / 24.0 us for S / T along x against 14.5 / 16.0 here,
-// but 15.4 against 29 for the fused pair), from 127^2 on these are (127^2: S 17.8 and 23.5 us along x and y
-// against 15; 511^2: 47 against 24, T 87 against 27; 255^3: S 2000 against 415, T 3870 against 475).  The
-// mixed form's residual products have double-float passes to beat: 255^3 860-970 against 480 us, but 511^2 33
+// FP64 form: a tile takes 8 us whatever its size, and the fused FFT passes are two launches each here, while an
+// FP64 FFT pass costs in proportion to the points.  A time step of the FP64 form (4 Arnoldi steps) with digit /
+// FFT passes: 127^2 0.52 / 0.40 ms, 255 x 127 0.55 / 0.43, 15 x 63 x 63 0.686 / 0.679, 255^2 0.58 / 0.60,
+// 511 x 255 0.72 / 1.04, 511^2 0.92 / 2.04, 127 x 63 x 127 1.80 / 7.01: they meet at 60000 points.
+// Mixed form: the residual products have double-float passes to beat: 255^3 860-970 against 480 us, but 511^2 33
 // against 27, and a batch of 16 grids of 127..511 points per axis took 24.9 ms with those and 25.9 with these
 // (a block here fills half an SM, so the instances' streams overlap less), hence from 2^20 points on.
-bool digit_context(const rfnse_ctx* c) { return c->d > 1 && c->N >= (c->p.precision == 1 ? 1 << 20 : 8192); }
+bool digit_context(const rfnse_ctx* c) { return c->d > 1 && c->N >= (c->p.precision == 1 ? 1 << 20 : 60000); }
 
 template <int FLAGS>
 cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s) {

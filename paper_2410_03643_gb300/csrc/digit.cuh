@@ -173,20 +173,35 @@ cudaError_t launch_digit_form(rfnse_ctx* c, const PassParams& p, int axis, int h
   return e;
 }
 
-// One pass of the solver along `axis`: the digit form where it pays (or where the tuner found it fastest), the
-// line pass otherwise.  To the tuner the digit form is one more geometry (variant 2) of the configuration.
+// Geometry of an FP64 line pass without tuning: the default tile, halved while that leaves fewer than two
+// blocks per SM.  A block's FFTs are bound by its SM's FP64 pipe (2 operations per cycle: eight lines of 64 points
+// took 9 us), so on a small grid every line goes to an SM of its own.
+template <int FLAGS>
+PassGeom fp64_pass_geometry(const PassParams& p) {
+  PassGeom g = default_pass_geometry<FLAGS>(p, false);
+  auto blocks = [&](int B) {
+    return p.stride == 1 ? (p.nlines + B - 1) / B : ((p.stride + B - 1) / B) * (p.nlines / p.stride);
+  };
+  while (g.B > 1 && blocks(g.B) < 2 * 152) g.B >>= 1;
+  return g;
+}
+
+// One pass of the solver along `axis`: the digit form where the context has its tables (or where the tuner found
+// it fastest), the line pass otherwise.  To the tuner the digit form is one more geometry (variant 2).
 template <typename R, typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
 cudaError_t solver_pass(rfnse_ctx* c, const PassParams& p, int axis, int half, cudaStream_t s) {
-  if constexpr (!digit_form<R, TIN, TOUT, TACCI, TACCO, FLAGS>()) {
+  constexpr bool form = digit_form<R, TIN, TOUT, TACCI, TACCO, FLAGS>();
+  const bool possible = form && (sizeof(R) == 8 ? digit_possible(c, axis) : digit32_possible(c, axis));
+  if (c->param_rec || (sizeof(R) == 4 && !possible)) {
     return launch_pass<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s);
   } else {
-    const bool possible = sizeof(R) == 8 ? digit_possible(c, axis) : digit32_possible(c, axis);
-    if (c->param_rec || !possible) return launch_pass<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s);
     auto launch = [c, p, axis, half, s](const PassGeom& g) {
-      return g.variant == 2 ? launch_digit_form<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, axis, half, s)
-                            : launch_pass_geom<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s, g);
+      if constexpr (form) {
+        if (g.variant == 2) return launch_digit_form<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, axis, half, s);
+      }
+      return launch_pass_geom<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, s, g);
     };
-    PassGeom g{1, 1, 2};
+    PassGeom g = possible ? PassGeom{1, 1, 2} : fp64_pass_geometry<FLAGS>(p);
     if (c->tune_rec || !c->tune.empty()) {
       const unsigned long long key = pass_key<R, TIN, TOUT, TACCI, TACCO, FLAGS>(c, p);
       if (c->tune_rec) {  // rfnse_autotune is recording the solver's pass configurations

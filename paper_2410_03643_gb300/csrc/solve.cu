@@ -781,10 +781,16 @@ rfnse_status autotune(rfnse_ctx* c, int reps, int force, int* n_configs, int* n_
       std::lock_guard<std::mutex> lock(g_tune_mutex);
       const auto it = g_tune_memo.find(mk);
       if (it != g_tune_memo.end()) {
+        // a choice of a context with other kernels (digit tables or none) does not apply here
+        auto same = [&](const PassGeom& g) {
+          return g.B == it->second.first.B && g.nt == it->second.first.nt && g.variant == it->second.first.variant;
+        };
+        have = same(r.dflt) || std::any_of(r.cands.begin(), r.cands.end(), same);
+      }
+      if (have) {
         best = it->second.first;
         tb = g_tune_times[mk].first;
         td = g_tune_times[mk].second;
-        have = true;
       }
     }
     if (!have) {

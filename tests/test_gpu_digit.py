@@ -36,12 +36,12 @@ def _matrices(p, axis):
     return S, mu * np.array(c)[np.abs(j[:, None] - j[None, :])]
 
 
-@pytest.mark.parametrize("n", [(255, 63), (127, 127), (511, 31), (31, 511), (3, 7, 511), (7, 255, 15), (63, 15, 31)])
+@pytest.mark.parametrize("n", [(255, 255), (511, 127), (127, 511), (3, 127, 255), (7, 255, 63), (63, 15, 127), (31, 63, 31)])
 def test_digit_passes_match_the_matrices(n):
     from paper_2410_03643_gb300 import Solver
     d = len(n)
     p = W.Problem(d=d, n=n, lo=(-8.0,) * d, hi=(8.0,) * d, alpha=1.5, rho=1.0, dt=0.005)
-    assert p.size >= 8192
+    assert p.size >= 60000
     s = Solver(p, precision=0)
     x = W.random_field(p.shape, 7)
     x.reshape(-1)[:: 97] *= 1e6                      # lines of very uneven magnitude
@@ -63,7 +63,7 @@ def test_digit_passes_match_the_matrices(n):
 def test_digit_passes_at_the_ends_of_the_number_range():
     """A zero line, subnormal and huge lines, and one line with an infinity: only that line is NaN."""
     from paper_2410_03643_gb300 import Solver
-    p = W.Problem(d=2, n=(255, 63), lo=(-8.0, -8.0), hi=(8.0, 8.0), alpha=1.5, rho=1.0, dt=0.005)
+    p = W.Problem(d=2, n=(255, 255), lo=(-8.0, -8.0), hi=(8.0, 8.0), alpha=1.5, rho=1.0, dt=0.005)
     s = Solver(p, precision=0)
     x = W.random_field(p.shape, 9)
     x[0] = 0
@@ -73,7 +73,7 @@ def test_digit_passes_at_the_ends_of_the_number_range():
     x[4, 0] = complex(0.0, np.nan)
     y = s.dst(0, torch.from_numpy(x.reshape(-1).copy()).cuda()).cpu().numpy().reshape(p.shape)
     S, _ = _matrices(p, 0)
-    ok = [r for r in range(63) if r not in (3, 4)]
+    ok = [r for r in range(255) if r not in (3, 4)]
     assert np.all(y[0] == 0)
     assert not np.any(np.isfinite(y[3].real)) and not np.any(np.isfinite(y[4].imag))
     for r in ok[2:]:
