@@ -335,7 +335,7 @@ int rfnse_create(const rfnse_params* p, void* stream, rfnse_ctx** out) {
   chk(dalloc(&c->partials, 1024));
   chk(dalloc(&c->counter, 1));
   chk(dalloc(&c->gs, 1));
-  if (e == cudaSuccess) chk(host_alloc_pinned((void**)&c->peek, sizeof(GmresPeek)));
+  if (e == cudaSuccess) chk(host_alloc_pinned((void**)&c->peek, 2 * sizeof(GmresPeek)));
   if (e != cudaSuccess) {
     g_create_error = std::string("allocation failed: ") + cudaGetErrorString(e);
     cudaGetLastError();

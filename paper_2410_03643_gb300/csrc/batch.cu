@@ -425,16 +425,6 @@ cudaError_t build_lockstep_graph(rfnse_batch* b, int v) {
 
 bool steady(const rfnse_ctx* c) { return c->step >= 1 && (c->p.precision == 0 || c->tu_valid[c->iprev]); }
 
-// Kernels one captured solve executed, from its statistics (as counted for stand-alone solves).
-long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk) {
-  const int d = c->d;
-  const int mixed = c->p.precision == 1;
-  const long long step_k = (d == 1 ? 1 : 3 * d - 2) + 1;
-  const long long cycle_k = mixed ? 1 + 1 + d + 1 + 1 : 1 + 1 + 1 + (d == 1 ? 1 : 2 * d - 1) + d + 1;
-  const long long cycles = mixed ? pk.outer : (pk.it > 0 ? pk.outer + 1 : 0);
-  return 2 + step_k * pk.it + cycle_k * cycles;
-}
-
 thread_local std::string g_batch_create_error;
 
 constexpr int kLockstepMinCount = 8;  // batches of at least this many eligible instances start in lock-step
@@ -555,11 +545,19 @@ int rfnse_batch_run(rfnse_batch* b, int nsteps, int* iters, double* relres) {
     // a failing instance does not stop the others' step: every instance takes this step (or fails it),
     // then the first failure is reported
     int fail = RFNSE_OK;
-    if (!all_steady) {  // first steps: every instance on its own (host-driven) until all are steady
+    if (!all_steady) {  // first steps: every instance on its own until all are steady.  Where the solves are
+                        // graphs all instances' steps are enqueued, each on its stream, before the first is
+                        // waited for (a batch of 16 grids of 127..511 points per axis spent 17 of the 25 ms of
+                        // its first five steps on solves one after another)
+      std::vector<int> queued(b->count, -1);  // status of the enqueued part; -1: not enqueued
+      for (int i = 0; i < b->count; ++i)
+        if (b->ctx[i]->use_graphs) queued[i] = time_step_enqueue(b->ctx[i]);
       for (int i = 0; i < b->count; ++i) {
         int it = 0;
         double rr = 0.0;
-        const int st = rfnse_run(b->ctx[i], 1, nullptr, &it, &rr, 1);
+        int st = queued[i];
+        if (st < 0) st = rfnse_run(b->ctx[i], 1, nullptr, &it, &rr, 1);
+        else if (st == RFNSE_OK) st = time_step_finish(b->ctx[i], &it, &rr);
         if (st != RFNSE_OK && st != RFNSE_ENOCONV && fail == RFNSE_OK) {
           b->err = "instance " + std::to_string(i) + ": " + rfnse_last_error(b->ctx[i]);
           fail = st;

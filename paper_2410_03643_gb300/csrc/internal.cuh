@@ -309,7 +309,8 @@ struct rfnse_ctx {
   unsigned* counter = nullptr;
   int red_blocks = 1;
   rfnse::GmresState* gs = nullptr;
-  rfnse::GmresPeek* peek = nullptr;  // pinned host
+  rfnse::GmresPeek* peek = nullptr;  // pinned host: the statistics of a time step's solves (two)
+  int pending = 0;                   // solves of the step in flight (time_step_enqueue)
   // device-side control: cooperative Arnoldi kernel and one CUDA graph per (precision, half)
   rfnse::GridBarrier* bar = nullptr;
   double* coop_partials = nullptr;   // 2 * coop_blocks

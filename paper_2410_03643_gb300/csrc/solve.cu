@@ -503,9 +503,25 @@ static cudaError_t build_solve_graph(rfnse_ctx* c, int mixed, int half) {
   return cudaSuccess;
 }
 
-// Solve R x = f on the device loop; f, x may be any buffers (copied to / from the graph's own).
-static rfnse_status solve_graph(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
-                                double* relres, int* outer_out) {
+// Kernels a solve graph executed: 2 at the start, per Arnoldi step its passes and the MGS kernel, per cycle
+// the cycle start, back-substitution, update and residual kernels.
+long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk) {
+  const int mixed = c->p.precision == 1 ? 1 : 0, d = c->d;
+  // a digit form makes two launches of the DST-Lambda-DST pass and of the fused x pass
+  auto digit_k = [&](int axis) {
+    return c->p.precond == 0 && c->tune.empty() && (mixed ? digit32_possible(c, axis) : digit_possible(c, axis)) ? 1 : 0;
+  };
+  const int lam_k = d > 1 ? digit_k(d - 1) : 0, fused_k = d > 1 ? digit_k(0) : 0;
+  const long long step_k = (d == 1 ? 1 : 3 * d - 2) + lam_k + fused_k + 1;
+  const long long cycle_k = mixed ? 1 + 1 + d + 1 + 1 : 1 + 1 + 1 + (d == 1 ? 1 : 2 * d - 1) + lam_k + d + 1;
+  const long long cycles = mixed ? pk.outer : (pk.it > 0 ? pk.outer + 1 : 0);
+  return 2 + step_k * pk.it + cycle_k * cycles;
+}
+
+// Enqueue the solve of R x = f on the device loop, its statistics going to c->peek[slot]; f, x may be any
+// buffers (copied to / from the graph's own).
+static rfnse_status solve_graph_enqueue(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half,
+                                        int slot) {
   const int mixed = c->p.precision == 1 ? 1 : 0;
   const int h = half ? 1 : 0;
   const long long N = c->N;
@@ -516,25 +532,17 @@ static rfnse_status solve_graph(rfnse_ctx* c, const double* D, const double2* f,
   c->tables_ready = false;
   RFNSE_CUDA_TRY(c, cudaGraphLaunch(c->graph_exec[mixed][h], c->stream));
   if (x != c->x) RFNSE_CUDA_TRY(c, cudaMemcpyAsync(x, c->x, sizeof(double2) * N, cudaMemcpyDeviceToDevice, c->stream));
-  GmresPeek pk;
-  rfnse_status st = peek(c, &pk);
-  if (st) return st;
+  RFNSE_CUDA_TRY(c, cudaMemcpyAsync(c->peek + slot, c->gs, sizeof(GmresPeek), cudaMemcpyDeviceToHost, c->stream));
+  return RFNSE_OK;
+}
+
+// What an enqueued solve came to, once the stream has been waited for.
+static rfnse_status solve_graph_status(rfnse_ctx* c, const GmresPeek& pk, int* iters, double* relres, int* outer_out) {
+  const int mixed = c->p.precision == 1 ? 1 : 0;
   *iters = pk.it;
   *relres = pk.relres;
   *outer_out = pk.outer;
-  {  // kernels the graph executed: 2 at the start, per Arnoldi step its passes and the MGS kernel,
-     // per cycle the cycle start, back-substitution, update and residual kernels
-    const int d = c->d;
-    // a digit form makes two launches of the DST-Lambda-DST pass and of the fused x pass
-    auto digit_k = [&](int axis) {
-      return c->p.precond == 0 && c->tune.empty() && (mixed ? digit32_possible(c, axis) : digit_possible(c, axis)) ? 1 : 0;
-    };
-    const int lam_k = d > 1 ? digit_k(d - 1) : 0, fused_k = d > 1 ? digit_k(0) : 0;
-    const long long step_k = (d == 1 ? 1 : 3 * d - 2) + lam_k + fused_k + 1;
-    const long long cycle_k = mixed ? 1 + 1 + d + 1 + 1 : 1 + 1 + 1 + (d == 1 ? 1 : 2 * d - 1) + lam_k + d + 1;
-    const long long cycles = mixed ? pk.outer : (pk.it > 0 ? pk.outer + 1 : 0);
-    count_launch(2 + step_k * pk.it + cycle_k * cycles);
-  }
+  count_launch(solve_kernels(c, pk));
   c->resid_current = mixed && pk.outer > 0;
   if (pk.err) { c->err = "a bounded device-side wait gave up"; return RFNSE_ETIMEOUT; }
   if (pk.done == 3) { c->err = "non-finite value in the solve"; return RFNSE_ENUMERIC; }
@@ -542,6 +550,14 @@ static rfnse_status solve_graph(rfnse_ctx* c, const double* D, const double2* f,
   if (pk.done == 1 || pk.done == 2) return RFNSE_OK;
   c->err = mixed ? "mixed-precision refinement did not reach tol" : "GMRES reached max_it";
   return RFNSE_ENOCONV;
+}
+
+static rfnse_status solve_graph(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
+                                double* relres, int* outer_out) {
+  const rfnse_status st = solve_graph_enqueue(c, D, f, x, half, 0);
+  if (st) return st;
+  RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return solve_graph_status(c, c->peek[0], iters, relres, outer_out);
 }
 
 rfnse_status solve_block(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
@@ -619,7 +635,74 @@ static void keep_Tu(rfnse_ctx* c, rfnse_status st, const double* D, const double
   }
 }
 
+// The step with its solves as graphs, in two halves: nothing in it needs the host between its solves (a
+// predictor that fails leaves the corrector nothing finite to do), so a whole step is enqueued and then waited
+// for, and a batch enqueues every instance's step first.
+rfnse_status time_step_enqueue(rfnse_ctx* c) {
+  const long long N = c->N;
+  const int inext = 3 - c->iprev - c->icur;
+  double2* un = c->u[inext];
+  rfnse_status st;
+  c->tu_valid[inext] = false;
+  c->pending = 0;
+  if (c->step == 0) {
+    const double2* u0 = c->u[c->icur];
+    const double rdt = c->p.rho * c->p.dt * 0.5;
+    launch_diag(u0, nullptr, c->D, rdt, N, c->stream);
+    RFNSE_CUDA_TRY(c, run_matvec_fp64(c, u0, c->D, c->f, nullptr, kOne, kMinusI, 1, nullptr));
+    if ((st = solve_graph_enqueue(c, c->D, c->f, un, 1, 0)) != RFNSE_OK) return st;
+    c->pending = 1;
+    if (c->p.first_step == 1) {
+      if (c->keep_pred)  // the reverse pass reads the predictor
+        RFNSE_CUDA_TRY(c, cudaMemcpyAsync(c->keep_pred, un, sizeof(double2) * N, cudaMemcpyDeviceToDevice, c->stream));
+      launch_diag(u0, un, c->D, rdt, N, c->stream);
+      RFNSE_CUDA_TRY(c, run_matvec_fp64(c, u0, c->D, c->f, nullptr, kOne, kMinusI, 1, nullptr));
+      if ((st = solve_graph_enqueue(c, c->D, c->f, un, 1, 1)) != RFNSE_OK) return st;
+      c->pending = 2;
+    }
+  } else {
+    const double2* up = c->u[c->iprev];
+    const double2* uc = c->u[c->icur];
+    if (c->tu_valid[c->iprev]) {  // mixed form: D, f and the sub-solve tables in one sweep
+      launch_step_prep(c, uc, up, c->Tu[c->iprev], c->stream);
+      c->tables_ready = true;
+    } else {
+      launch_diag(uc, nullptr, c->D, c->p.rho * c->p.dt, N, c->stream);
+      RFNSE_CUDA_TRY(c, run_matvec_fp64(c, up, c->D, c->f, nullptr, kOne, kMinusI, 0, nullptr));
+    }
+    if ((st = solve_graph_enqueue(c, c->D, c->f, un, 0, 0)) != RFNSE_OK) return st;
+    c->pending = 1;
+  }
+  return RFNSE_OK;
+}
+
+rfnse_status time_step_finish(rfnse_ctx* c, int* iters, double* relres) {
+  NvtxRange range("rfnse solve");
+  RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  const int inext = 3 - c->iprev - c->icur;
+  rfnse_status st = RFNSE_OK;
+  int it = 0;
+  for (int q = 0; q < c->pending; ++q) {
+    int iq = 0, outer = 0;
+    const rfnse_status sq = solve_graph_status(c, c->peek[q], &iq, relres, &outer);
+    c->last_outer = outer;
+    if (sq != RFNSE_OK && sq != RFNSE_ENOCONV) return sq;
+    if (sq != RFNSE_OK) st = sq;
+    it += iq;
+  }
+  keep_Tu(c, st, c->D, c->f, inext, c->step == 0 ? 2.0 : 1.0);  // the first step's system has T/2
+  c->iprev = c->icur;
+  c->icur = inext;
+  c->step += 1;
+  *iters = it;
+  return st;
+}
+
 rfnse_status time_step(rfnse_ctx* c, int* iters, double* relres) {
+  if (c->use_graphs) {
+    const rfnse_status st = time_step_enqueue(c);
+    return st != RFNSE_OK ? st : time_step_finish(c, iters, relres);
+  }
   const long long N = c->N;
   const int inext = 3 - c->iprev - c->icur;
   double2* un = c->u[inext];

@@ -15,8 +15,14 @@ cudaError_t run_apply_A(rfnse_ctx* c, const double2* u, double2* out, const doub
 rfnse_status solve_block(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
                          double* relres);
 rfnse_status time_step(rfnse_ctx* c, int* iters, double* relres);
+// the two halves of a time step of a context whose solves are graphs (c->use_graphs): enqueue it on the
+// context's stream, and wait for it; between them other contexts' steps can be enqueued
+rfnse_status time_step_enqueue(rfnse_ctx* c);
+rfnse_status time_step_finish(rfnse_ctx* c, int* iters, double* relres);
 rfnse_status tban_solve(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
                         double* relres);
+// kernels one solve graph executed, from its statistics
+long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk);
 cudaError_t prepare_D(rfnse_ctx* c, const double* D);
 // f_part / f_n: block partials of ||f||^2 left by f's producer in the same graph (f_n = 0: none)
 // the settings of c's solves (mixed = 1: the mixed form)
