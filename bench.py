@@ -91,6 +91,21 @@ KERNEL_CLASSES = {
     "df_toep_acc": (1024 | 32, "hbm", "k_toeplitz_df<F_TOEP_ACC> (residual Toeplitz y / z, double-float FFTs)",
                     _DF_SRC),
 }
+# The 3-D workload (2^20 points and more) runs these classes as tensor-core digit passes, some of them two
+# launches: its descriptions and sources.
+_DIG_SRC = ("digit.cu", "digit.cuh", "tc05.cuh")
+_DIG32_SRC = ("digit32.cu", "digit.cuh", "tc05.cuh")
+CLASSES_3D = {
+    "fp32_fused_x": ("k_digit32<F_DST|F_DSCALE>, k_digit32<F_TOEP_X> (inverse S x + (wI+D) sub-solve; Toeplitz x)",
+                     _DIG32_SRC),
+    "fp32_dst": ("line pass <float, F_INSCALE|F_DST> (S x with the Arnoldi scaling folded in), k_digit32<F_DST> (S y)",
+                 _DIG32_SRC + _PASS_SRC),
+    "fp32_dst_lam": ("k_digit32<F_DST|F_LAM>, k_digit32<F_DST> (S, divide by (w + i Lambda); S; last axis)",
+                     _DIG32_SRC),
+    "fp32_toep_acc": ("k_digit32<F_TOEP_ACC> (Toeplitz y / z, accumulated)", _DIG32_SRC),
+    "df_toep_x": ("k_digit<F_TOEP_X> (residual Toeplitz x, FP64 digits)", _DIG_SRC),
+    "df_toep_acc": ("k_digit<F_TOEP_ACC> (residual Toeplitz y / z, FP64 digits)", _DIG_SRC),
+}
 PROFILED = {
     "2d": ("arnoldi", "fp32_fused_x", "fp32_dst", "fp32_dst_lam", "fp32_toep_acc", "df_toep_x", "df_toep_acc"),
     "3d": ("arnoldi", "fp32_fused_x", "fp32_dst", "fp32_dst_lam", "fp32_toep_acc", "df_toep_x", "df_toep_acc"),
@@ -110,13 +125,13 @@ TRAFFIC = {
     ("2d", "fp32_toep_acc"): (8398976, "bc9364c29794"),
     ("2d", "df_toep_x"): (6342912, "dcc06e68e64c"),
     ("2d", "df_toep_acc"): (8433408, "dcc06e68e64c"),
-    ("3d", "arnoldi"): (1813218440, "2f0ff00eb74a"),
-    ("3d", "fp32_fused_x"): (555763840, "bc9364c29794"),
-    ("3d", "fp32_dst"): (349960619, "bc9364c29794"),
-    ("3d", "fp32_dst_lam"): (370098944, "bc9364c29794"),
-    ("3d", "fp32_toep_acc"): (422121472, "bc9364c29794"),
-    ("3d", "df_toep_x"): (880270336, "dcc06e68e64c"),
-    ("3d", "df_toep_acc"): (756481408, "dcc06e68e64c"),
+    ("3d", "arnoldi"): (1280290602, "2f0ff00eb74a"),
+    ("3d", "fp32_fused_x"): (653813546, "8c52addd920e"),
+    ("3d", "fp32_dst"): (340754232, "ead6a498f30a"),
+    ("3d", "fp32_dst_lam"): (568991829, "8c52addd920e"),
+    ("3d", "fp32_toep_acc"): (550711232, "8c52addd920e"),
+    ("3d", "df_toep_x"): (765149120, "8d048f9dab6e"),
+    ("3d", "df_toep_acc"): (749146709, "8d048f9dab6e"),
 }
 
 
@@ -135,7 +150,8 @@ def traffic_for(workload_name: str, cls: str):
     if rec is None:
         return None, "no ncu capture of this class on this workload"
     value, digest = rec
-    if digest != source_digest(KERNEL_CLASSES[cls][3]):
+    srcs = CLASSES_3D[cls][1] if workload_name == "3d" and cls in CLASSES_3D else KERNEL_CLASSES[cls][3]
+    if digest != source_digest(srcs):
         return None, "stale: the kernel's sources changed since the ncu capture"
     return value, "ncu dram__bytes_read.sum + dram__bytes_write.sum per launch"
 
@@ -437,6 +453,8 @@ def roofline_entry(name: str, cls: str, prof, ms_serial: float, nprof: int):
     algorithmic flops, algorithmic bytes)."""
     n, pms, fl, by = prof
     kind, bound, desc, _ = KERNEL_CLASSES[cls]
+    if name == "3d" and cls in CLASSES_3D:
+        desc = CLASSES_3D[cls][0]
     hbm, how = measured_hbm_gbs()
     traffic, tnote = traffic_for(name, cls)
     gbs = by / (pms * 1e-3) / 1e9

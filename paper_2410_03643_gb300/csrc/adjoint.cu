@@ -326,6 +326,7 @@ int rfnse_tape_backward(rfnse_ctx* c, const void* gN, void* g0, double* grho, in
   RFNSE_CUDA_TRY(c, cudaMemcpyAsync(&acc, c->adj_red + kAdjMaxBlocks, sizeof(double), cudaMemcpyDeviceToHost,
                                     c->stream));
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  if (const rfnse_status sd = digit_status(c)) return sd;
   if (grho) *grho = acc;
   if (iters) *iters = total_it;
   // leave the context at the taped run's final state

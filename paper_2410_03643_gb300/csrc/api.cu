@@ -335,13 +335,14 @@ int rfnse_create(const rfnse_params* p, void* stream, rfnse_ctx** out) {
   chk(dalloc(&c->partials, 1024));
   chk(dalloc(&c->counter, 1));
   chk(dalloc(&c->gs, 1));
-  if (e == cudaSuccess) chk(host_alloc_pinned((void**)&c->peek, 2 * sizeof(GmresPeek)));
+  if (e == cudaSuccess) chk(host_alloc_pinned((void**)&c->peek, 3 * sizeof(GmresPeek)));
   if (e != cudaSuccess) {
     g_create_error = std::string("allocation failed: ") + cudaGetErrorString(e);
     cudaGetLastError();
     free_ctx(c);
     return (e == cudaErrorMemoryAllocation) ? RFNSE_ENOMEM : RFNSE_ECUDA;
   }
+  std::memset(c->peek, 0, 3 * sizeof(GmresPeek));
   chk(cudaMemsetAsync(c->counter, 0, sizeof(unsigned), c->stream));
   chk(cudaMemsetAsync(c->gs, 0, sizeof(GmresState), c->stream));
   chk(cudaMemsetAsync(c->bar, 0, sizeof(GridBarrier), c->stream));
@@ -494,14 +495,14 @@ int rfnse_apply_A(rfnse_ctx* c, const void* u, void* out, const double* D, int h
   if (!c || !u || !out || !D || u == out) return RFNSE_EINVAL;
   RFNSE_CUDA_TRY(c, run_apply_A(c, (const double2*)u, (double2*)out, D, half ? 1 : 0));
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return RFNSE_OK;
+  return digit_status(c);
 }
 
 int rfnse_apply_prec(rfnse_ctx* c, const void* v, void* z, const double* D, int half, int precision) {
   if (!c || !v || !z || !D || v == z || (precision != 0 && precision != 1)) return RFNSE_EINVAL;
   RFNSE_CUDA_TRY(c, run_apply_prec(c, (const double2*)v, (double2*)z, D, half ? 1 : 0, precision));
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return RFNSE_OK;
+  return digit_status(c);
 }
 
 int rfnse_dst(rfnse_ctx* c, int axis, const void* in, void* out, int precision) {
@@ -509,14 +510,14 @@ int rfnse_dst(rfnse_ctx* c, int axis, const void* in, void* out, int precision) 
     return RFNSE_EINVAL;
   RFNSE_CUDA_TRY(c, run_dst(c, axis, (const double2*)in, (double2*)out, precision));
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return RFNSE_OK;
+  return digit_status(c);
 }
 
 int rfnse_toeplitz(rfnse_ctx* c, int axis, const void* in, void* out, int half) {
   if (!c || !in || !out || in == out || axis < 0 || axis >= c->d) return RFNSE_EINVAL;
   RFNSE_CUDA_TRY(c, run_toeplitz(c, axis, (const double2*)in, (double2*)out, half ? 1 : 0));
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return RFNSE_OK;
+  return digit_status(c);
 }
 
 int rfnse_solve(rfnse_ctx* c, const double* D, const void* b, void* u, int half, int* iters, double* relres) {

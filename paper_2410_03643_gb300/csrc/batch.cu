@@ -617,7 +617,7 @@ int rfnse_batch_run(rfnse_batch* b, int nsteps, int* iters, double* relres) {
       c->tu_valid[v] = false;
       if (iters) iters[(size_t)s * b->count + i] = pk.it;
       if (relres) relres[(size_t)s * b->count + i] = pk.relres;
-      if (pk.err && fail == RFNSE_OK) {
+      if ((digit_status(c) != RFNSE_OK || pk.err) && fail == RFNSE_OK) {
         b->err = "instance " + std::to_string(i) + ": a bounded device-side wait gave up";
         fail = RFNSE_ETIMEOUT;
       }

@@ -90,6 +90,11 @@ __device__ __forceinline__ double2 coef_times(int code, double2 c, double2 v) {
 }
 
 // KB: K / 128 of a half; FOLD: sums and differences (two halves), else stacked whole lines.
+// 255^3, S 2000 -> 415 us, T 3870 -> 480 us (the FP64 FFT passes before, these now); 511^2, S 47 -> 24 us, T 87 -> 27.
+// Nothing is saturated (255 x 255 x 63, S: ALU pipe 49%, tensor 24%, L2 17% of peak; T also FP64 23%): two blocks
+// per SM, all that TMEM holds, take turns at the integer work of the digits (4000 cycles of a tile of 16 lines
+// and one half), the products (6400), the sums (2100) and the results (3000, T 7600 with the exchange of the halves).
+// 512 threads of one part each against 256 of both: 415 against 438 us.  Folding in FP64 instead of integers: 494.
 template <int FLAGS, int KB, bool FOLD>
 __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassParams p, const DigitArgs a) {
   constexpr bool TOEP = (FLAGS & (F_TOEP_X | F_TOEP_ACC)) != 0;
@@ -539,7 +544,7 @@ cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream
   a.ca_code = coef_code(p.ca);
   a.cb_code = coef_code(p.cb);
   a.lam_scale = 1.0 / p.dst_scale;
-  a.err = &c->gs->err;
+  a.err = &c->peek[2].err;  // pinned: written by the kernel only when a wait gives up
   const long long per = (long long)kDigLines * sh.stack;
   long long tiles;
   if (p.stride == 1) {

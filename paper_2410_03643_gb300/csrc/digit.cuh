@@ -75,9 +75,10 @@ bool digit_possible(const rfnse_ctx* c, int axis);
 template <int FLAGS>
 cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s);
 
-// The FP32 passes of the mixed form: whether an axis has them, and one pass with the given storage types.
+// The FP32 passes of the mixed form: whether an axis has them, and one pass with the given storage types (input
+// in FP32).
 bool digit32_possible(const rfnse_ctx* c, int axis);
-template <typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
+template <typename TOUT, typename TACCI, typename TACCO, int FLAGS>
 cudaError_t run_digit32(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s);
 
 // The passes that have a digit form: a sine transform or a Toeplitz product, and not the fused pass of 1-D
@@ -90,7 +91,7 @@ constexpr bool digit_form() {
   constexpr bool in16 = sizeof(TIN) == 16, out16 = sizeof(TOUT) == 16, ai16 = sizeof(TACCI) == 16,
                  ao16 = sizeof(TACCO) == 16;
   if (sizeof(R) == 8) return in16 && out16 && ai16 && ao16;
-  if (out16 || in16 != ((FLAGS & F_INSCALE) != 0)) return false;
+  if (out16 || in16) return false;
   if (FLAGS & F_DSCALE) return (FLAGS & F_TOEP_X) && !(FLAGS & F_DOT0) && ai16 && !ao16;
   if (FLAGS & F_DST) return ai16 && ao16;
   return (FLAGS & F_TOEP_ACC) && !ai16 && (ao16 || !(FLAGS & F_DOT0));
@@ -99,7 +100,7 @@ constexpr bool digit_form() {
 template <typename R, typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
 cudaError_t run_digit_any(rfnse_ctx* c, const PassParams& p, int axis, int half, cudaStream_t s) {
   if constexpr (sizeof(R) == 8) return run_digit<FLAGS>(c, p, axis, half, s);
-  else return run_digit32<TIN, TOUT, TACCI, TACCO, FLAGS>(c, p, axis, half, s);
+  else return run_digit32<TOUT, TACCI, TACCO, FLAGS>(c, p, axis, half, s);
 }
 
 // CUDA events around the launches of a profiled pass (rfnse_profile): the stop event, null when the pass

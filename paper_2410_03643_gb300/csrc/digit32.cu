@@ -12,7 +12,11 @@
 // streamed through shared memory for every tile, was bound by that stream at 60 B per cycle and SM (157 and
 // 249 us).  So a block stays on its SM, keeps the operator in TMEM (five of its six digit blocks, the sixth in
 // shared memory) and runs its tiles through two roles at once: two groups of warps read lines, split them into
-// digits and issue the products (alternate tiles), one group drains the accumulators and does the pointwise work.
+// digits and issue the products (alternate tiles), one group drains the accumulators and does the pointwise work,
+// which bounds the passes now.  255^3, us (bytes over time in TB/s) before and after: S 125 -> 72 (3.7), S / (w + i
+// Lambda) and S together 230 -> 191, S with the sub-solve and T_x 300 -> 217, T 227 -> 114 (3.5), T with the
+// first Gram-Schmidt dot product 236 (3.4).  The pass that also scales and stores the FP64 basis vector stays an
+// FFT pass: it is bound by the FP64 products of that (148 us against 156).
 #include <cuda_fp16.h>
 #include <cmath>
 #include "digit.cuh"
@@ -51,17 +55,6 @@ static_assert(kStage % 16 == 0 && kOperS % 128 == 0, "alignment");
 
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kGroup) : "memory"); }
 
-// FP64 -> FP32 to nearest by integer operations (the FP64 pipe converts two values per cycle and SM);
-// below FP32's normal range 0, above it infinity, NaN kept.
-__device__ __forceinline__ float narrow(double v) {
-  const uint32_t hi = (uint32_t)__double2hiint(v), lo = (uint32_t)__double2loint(v);
-  const uint32_t e = (hi >> 20) & 0x7ff;
-  uint32_t r = (((hi & 0x7fffffffu) - 0x38000000u) << 3) | (lo >> 29);
-  r += (lo >> 28) & 1;
-  if (e <= 896) r = 0;
-  if (e >= 1151) r = e == 2047 && ((hi & 0xfffffu) | lo) ? 0x7fc00000u : 0x7f800000u;
-  return __uint_as_float(r | (hi & 0x80000000u));
-}
 // FP32 -> FP64, exact but for subnormal values (0), by integer operations
 __device__ __forceinline__ double widen(float v) {
   const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
@@ -70,7 +63,6 @@ __device__ __forceinline__ double widen(float v) {
   if (m >= 0x7f800000u) hi = 0x7ff00000u | ((m & 0x7fffffu) ? 0x80000u : 0u);
   return __hiloint2double((int)(hi | (b & 0x80000000u)), m >= 0x7f800000u ? 0 : (int)(m << 29));
 }
-__device__ __forceinline__ float2 get_c(const double2* p) { const double2 v = *p; return make_float2(narrow(v.x), narrow(v.y)); }
 __device__ __forceinline__ void put_c(double2* p, float2 v) { *p = make_double2(widen(v.x), widen(v.y)); }
 __device__ __forceinline__ void put_c(float2* p, float2 v) { *p = v; }
 
@@ -91,7 +83,7 @@ __device__ __forceinline__ void split2(float a, float b, uint32_t (&d)[kDigits32
   d[2] = pack(fmaf(u.x, -0x1p-11f, ra) * 0x1p22f, fmaf(u.y, -0x1p-11f, rb) * 0x1p22f);
 }
 
-template <typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS, bool FOLD>
+template <typename TOUT, typename TACCI, typename TACCO, int FLAGS, bool FOLD>
 __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Digit32Args a) {
   constexpr bool TOEP = (FLAGS & (F_TOEP_X | F_TOEP_ACC)) != 0;
   constexpr int HALVES = FOLD ? 2 : 1;
@@ -164,8 +156,8 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
     line0 = (xax ? tile : tile - hi * p.tiles_inner) * (kDigLines * a.stack);
     base0 = xax ? 0 : hi * p.stride * n;
   };
-  const TIN* in = reinterpret_cast<const TIN*>(p.in);
-  if (p.gdyn && p.in_dyn_z) in = reinterpret_cast<const TIN*>(p.zbase) + (long long)p.gdyn->j * p.ldv;
+  const float2* in = reinterpret_cast<const float2*>(p.in);
+  if (p.gdyn && p.in_dyn_z) in = reinterpret_cast<const float2*>(p.zbase) + (long long)p.gdyn->j * p.ldv;
   [[maybe_unused]] double dot = 0.0;
 
   if (uwarp < 16) {
@@ -175,17 +167,6 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
     auto slot_pos = [&](int i) { return xax ? i * 16 + kg : kg * 8 + i; };
     const bool mid = FOLD && 2 * slot_pos(7) == n - 1;  // the thread's last entry is the middle of the line
     unsigned char* dst0 = sm + kCtrl + grp * kBufBytes + kg * kLbo + ((2 * l) >> 3) * kSbo + ((2 * l) & 7) * 16;
-    [[maybe_unused]] double2* cpy = p.copy_out;
-    [[maybe_unused]] double sc = 1.0;
-    if constexpr ((FLAGS & F_INSCALE) != 0) {
-      if (p.gdyn) {
-        in = reinterpret_cast<const TIN*>(p.gdyn->src);
-        sc = p.gdyn->src_scale;
-        cpy = p.vbase + (long long)p.gdyn->j * p.ldv;
-      } else {
-        sc = *p.in_scale;
-      }
-    }
     const float2 zero = make_float2(0.0f, 0.0f);
     for (int k = grp; (long long)k * gridDim.x + blockIdx.x < a.tiles; k += 2) {
       long long base0, line0;
@@ -197,31 +178,10 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
         const long long g0 = base0 + (line0 + l) * lstep;
         const long long step = (xax ? 16 : 1) * estep;
         const long long ga = g0 + slot_pos(0) * estep, gb = g0 + (long long)(n - 1 - slot_pos(0)) * estep;
-        if constexpr ((FLAGS & F_INSCALE) != 0) {
 #pragma unroll
-          for (int q = 0; q < 8; q += 4) {  // in two parts, loads first: FP64 values take twice the registers
-            double2 x[4], y[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              x[i] = ok ? in[ga + (q + i) * step] : make_double2(0.0, 0.0);
-              y[i] = ok && !(q + i == 7 && mid) ? in[gb - (q + i) * step] : make_double2(0.0, 0.0);
-            }
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-              x[i] = cscale(x[i], sc);
-              y[i] = cscale(y[i], sc);
-              va[q + i] = make_float2(narrow(x[i].x), narrow(x[i].y));
-              vb[q + i] = make_float2(narrow(y[i].x), narrow(y[i].y));
-              if (ok) cpy[ga + (q + i) * step] = x[i];
-              if (ok && !(q + i == 7 && mid)) cpy[gb - (q + i) * step] = y[i];
-            }
-          }
-        } else {
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            va[i] = ok ? __ldg(reinterpret_cast<const float2*>(in) + ga + i * step) : zero;
-            vb[i] = ok && !(i == 7 && mid) ? __ldg(reinterpret_cast<const float2*>(in) + gb - i * step) : zero;
-          }
+        for (int i = 0; i < 8; ++i) {
+          va[i] = ok ? __ldg(in + ga + i * step) : zero;
+          vb[i] = ok && !(i == 7 && mid) ? __ldg(in + gb - i * step) : zero;
         }
       } else {
 #pragma unroll
@@ -230,16 +190,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
           const int sl = q >> a.log2N, pos = q - (sl << a.log2N);
           const long long ln = line0 + sl * kDigLines + l;
           const long long g = base0 + ln * lstep + pos * estep;
-          va[i] = zero;
-          if (ln < nline && pos < n) {
-            if constexpr ((FLAGS & F_INSCALE) != 0) {
-              const double2 x = cscale(in[g], sc);
-              cpy[g] = x;
-              va[i] = make_float2(narrow(x.x), narrow(x.y));
-            } else {
-              va[i] = __ldg(reinterpret_cast<const float2*>(in) + g);
-            }
-          }
+          va[i] = ln < nline && pos < n ? __ldg(in + g) : zero;
         }
       }
       unsigned m = 0;  // the line's largest magnitude
@@ -376,7 +327,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
             if (ok) op[q] = __ldg(reinterpret_cast<const float2*>(p.dfac) + g);
           }
           if constexpr ((FLAGS & F_TOEP_X) != 0) {
-            if (ok) op[q] = __ldg(reinterpret_cast<const float2*>(in) + g);
+            if (ok) op[q] = __ldg(in + g);
             if (ok && p.Dr) Dv[q] = __ldg(reinterpret_cast<const float*>(p.Dr) + g);
           }
           if constexpr ((FLAGS & F_TOEP_ACC) != 0) {
@@ -447,7 +398,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
             if constexpr ((FLAGS & F_TOEP_X) != 0) {
               y = csub(y, cscale(op[q], Dv[q]));
               acc = cmul(p.ca_f, op[q]);
-              if (p.acc_in) acc = cadd(acc, get_c(reinterpret_cast<const TACCI*>(p.acc_in) + g));
+              if (p.acc_in) acc = cadd(acc, to_c<float>(reinterpret_cast<const TACCI*>(p.acc_in)[g]));
             }
             acc = cadd(acc, cmul(p.cb_f, y));
             put_c(reinterpret_cast<TACCO*>(p.acc_out) + g, acc);
@@ -469,9 +420,9 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
   if constexpr ((FLAGS & F_DOT0) != 0) block_sum_store(dot, p.dot_part + blockIdx.x);
 }
 
-template <typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS, bool FOLD>
+template <typename TOUT, typename TACCI, typename TACCO, int FLAGS, bool FOLD>
 cudaError_t launch32(const PassParams& p, const Digit32Args& a, unsigned grid, cudaStream_t s) {
-  auto kern = k_digit32<TIN, TOUT, TACCI, TACCO, FLAGS, FOLD>;
+  auto kern = k_digit32<TOUT, TACCI, TACCO, FLAGS, FOLD>;
   static const cudaError_t attr = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (attr != cudaSuccess) return attr;
   count_launch();
@@ -483,7 +434,7 @@ cudaError_t launch32(const PassParams& p, const Digit32Args& a, unsigned grid, c
 
 bool digit32_possible(const rfnse_ctx* c, int axis) { return c->digS32[axis] != nullptr; }
 
-template <typename TIN, typename TOUT, typename TACCI, typename TACCO, int FLAGS>
+template <typename TOUT, typename TACCI, typename TACCO, int FLAGS>
 cudaError_t run_digit32(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream_t s) {
   constexpr bool TOEP = (FLAGS & (F_TOEP_X | F_TOEP_ACC)) != 0;
   DigitShape sh;
@@ -494,7 +445,7 @@ cudaError_t run_digit32(rfnse_ctx* c, PassParams p, int axis, int half, cudaStre
   a.log2N = p.log2L - 1;
   a.stack = sh.stack;
   a.lam_scale = (float)(1.0 / p.dst_scale);
-  a.err = &c->gs->err;
+  a.err = &c->peek[2].err;  // pinned: written by the kernel only when a wait gives up
   p.ca_f = make_float2((float)p.ca.x, (float)p.ca.y);
   p.cb_f = make_float2((float)p.cb.x, (float)p.cb.y);
   const long long per = (long long)kDigLines * sh.stack;
@@ -514,19 +465,18 @@ cudaError_t run_digit32(rfnse_ctx* c, PassParams p, int axis, int half, cudaStre
   if (e != cudaSuccess) return e;
   if (grid > sms) grid = sms;  // one block per SM, each over its share of the tiles
   if (FLAGS & F_DOT0) c->dot0_blocks = (int)grid;
-  if (sh.halves == 2) return launch32<TIN, TOUT, TACCI, TACCO, FLAGS, true>(p, a, (unsigned)grid, s);
-  return launch32<TIN, TOUT, TACCI, TACCO, FLAGS, false>(p, a, (unsigned)grid, s);
+  if (sh.halves == 2) return launch32<TOUT, TACCI, TACCO, FLAGS, true>(p, a, (unsigned)grid, s);
+  return launch32<TOUT, TACCI, TACCO, FLAGS, false>(p, a, (unsigned)grid, s);
 }
 
-#define RFNSE_DIGIT32(TI, TO, TAI, TAO, F) \
-  template cudaError_t run_digit32<TI, TO, TAI, TAO, F>(rfnse_ctx*, PassParams, int, int, cudaStream_t);
-RFNSE_DIGIT32(double2, float2, double2, double2, F_INSCALE | F_DST)
-RFNSE_DIGIT32(float2, float2, double2, double2, F_DST)
-RFNSE_DIGIT32(float2, float2, double2, double2, F_DST | F_LAM)
-RFNSE_DIGIT32(float2, float2, double2, float2, F_DST | F_DSCALE)
-RFNSE_DIGIT32(float2, float2, double2, float2, F_TOEP_X)
-RFNSE_DIGIT32(float2, float2, float2, float2, F_TOEP_ACC)
-RFNSE_DIGIT32(float2, float2, float2, double2, F_TOEP_ACC)
-RFNSE_DIGIT32(float2, float2, float2, double2, F_TOEP_ACC | F_DOT0)
+#define RFNSE_DIGIT32(TO, TAI, TAO, F) \
+  template cudaError_t run_digit32<TO, TAI, TAO, F>(rfnse_ctx*, PassParams, int, int, cudaStream_t);
+RFNSE_DIGIT32(float2, double2, double2, F_DST)
+RFNSE_DIGIT32(float2, double2, double2, F_DST | F_LAM)
+RFNSE_DIGIT32(float2, double2, float2, F_DST | F_DSCALE)
+RFNSE_DIGIT32(float2, double2, float2, F_TOEP_X)
+RFNSE_DIGIT32(float2, float2, float2, F_TOEP_ACC)
+RFNSE_DIGIT32(float2, float2, double2, F_TOEP_ACC)
+RFNSE_DIGIT32(float2, float2, double2, F_TOEP_ACC | F_DOT0)
 
 }  // namespace rfnse

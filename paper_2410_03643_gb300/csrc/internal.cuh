@@ -309,7 +309,8 @@ struct rfnse_ctx {
   unsigned* counter = nullptr;
   int red_blocks = 1;
   rfnse::GmresState* gs = nullptr;
-  rfnse::GmresPeek* peek = nullptr;  // pinned host: the statistics of a time step's solves (two)
+  // pinned host: the statistics of a time step's solves (two), and in the third's err what digit passes report
+  rfnse::GmresPeek* peek = nullptr;
   int pending = 0;                   // solves of the step in flight (time_step_enqueue)
   // device-side control: cooperative Arnoldi kernel and one CUDA graph per (precision, half)
   rfnse::GridBarrier* bar = nullptr;

@@ -134,11 +134,19 @@ cudaError_t run_apply_A(rfnse_ctx* c, const double2* u, double2* out, const doub
 
 // ---------------------------------------------------------------------------------------------
 
+rfnse_status digit_status(rfnse_ctx* c) {
+  volatile int* flag = &c->peek[2].err;
+  if (!*flag) return RFNSE_OK;
+  *flag = 0;
+  c->err = "a bounded device-side wait gave up";
+  return RFNSE_ETIMEOUT;
+}
+
 static rfnse_status peek(rfnse_ctx* c, GmresPeek* out) {
   RFNSE_CUDA_TRY(c, cudaMemcpyAsync(c->peek, c->gs, sizeof(GmresPeek), cudaMemcpyDeviceToHost, c->stream));
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   *out = *c->peek;
-  return RFNSE_OK;
+  return digit_status(c);
 }
 
 // ---- host loop -------------------------------------------------------------------------------
@@ -544,6 +552,7 @@ static rfnse_status solve_graph_status(rfnse_ctx* c, const GmresPeek& pk, int* i
   *outer_out = pk.outer;
   count_launch(solve_kernels(c, pk));
   c->resid_current = mixed && pk.outer > 0;
+  if (const rfnse_status sd = digit_status(c)) return sd;
   if (pk.err) { c->err = "a bounded device-side wait gave up"; return RFNSE_ETIMEOUT; }
   if (pk.done == 3) { c->err = "non-finite value in the solve"; return RFNSE_ENUMERIC; }
   if (pk.beta == 0.0 && pk.it == 0) { *relres = 0.0; return RFNSE_OK; }

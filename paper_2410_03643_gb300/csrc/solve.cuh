@@ -23,6 +23,8 @@ rfnse_status tban_solve(rfnse_ctx* c, const double* D, const double2* f, double2
                         double* relres);
 // kernels one solve graph executed, from its statistics
 long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk);
+// after the stream has been waited for: did a bounded wait of a digit pass give up since the last call?
+rfnse_status digit_status(rfnse_ctx* c);
 cudaError_t prepare_D(rfnse_ctx* c, const double* D);
 // f_part / f_n: block partials of ||f||^2 left by f's producer in the same graph (f_n = 0: none)
 // the settings of c's solves (mixed = 1: the mixed form)
