@@ -17,7 +17,7 @@ struct DigitArgs {
   int* err;                    // set when a bounded wait gives up
 };
 
-// Shared memory: barriers and line exponents, the vector's digits, the chunk ring.  The digits are one
+// Shared memory: barriers and line exponents (of every line stacked in a column), the vector's digits, the chunk ring.  The digits are one
 // K-major operand of 224 columns, digit j of column n at 32 j + n, because D_i .. D_6 are neighbours in
 // TMEM: for one operator digit a_i a single MMA of N = 32 (7 - i) columns forms its products with x_0 ..
 // x_{6-i}.  (An MMA costs 44 + N/2 cycles with A in shared memory, measured for N = 16..128: seven MMAs of
@@ -26,7 +26,8 @@ struct DigitArgs {
 // columns) and of an x pass (neighbouring entries, real and imaginary column) store without bank conflicts.
 constexpr int kSbo = 128, kLbo = kDigits * (kDigCols / 8) * kSbo + 32;
 constexpr int kDigitPitch = (kDigCols / 8) * kSbo;  // bytes from a digit to the next
-constexpr int kCtrl = 1024;
+constexpr int kCtrl = 128 + 32 * kDigLines * 4;  // up to 32 lines are stacked in each of the 16 columns
+static_assert(kCtrl % 128 == 0, "alignment");
 constexpr int kRowPitch = kDigLines * 16 + 16;  // staged results: a row's 16 lines, 16 B each
 template <int KB> constexpr int digit_bytes() { return (16 * KB * kLbo + 127) & ~127; }
 template <int KB> constexpr int digit_smem() { return kCtrl + digit_bytes<KB>() + kDigStages * kDigChunkBytes; }
@@ -136,7 +137,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       tc::mbar_init_fence();
       *s_fail = 0;
     }
-    if (lane < kDigLines) smax[lane] = 0;
+    for (int i = lane; i < kDigLines * a.stack; i += 32) smax[i] = 0;
     __syncwarp();
     tc::tmem_alloc(tc::smem_addr(s_tmem), COLS);
     tc::fence_before();
@@ -222,13 +223,13 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       }
     }
   }
-  {  // the column's largest exponent
+  // the largest exponent of each line: an exponent per stacked line (the operator is block diagonal, so the lines of
+  // a column need no common scale, and a tiny line beside a large or non-finite one keeps its digits)
+  if constexpr (FOLD) {
     unsigned m = 0;
 #pragma unroll
-    for (int i = 0; i < 8; ++i) {
-      m = max(m, (unsigned)__double2hiint(va[i]) & 0x7fffffffu);
-      if constexpr (FOLD) m = max(m, (unsigned)__double2hiint(vb[i]) & 0x7fffffffu);
-    }
+    for (int i = 0; i < 8; ++i)
+      m = max(m, max((unsigned)__double2hiint(va[i]) & 0x7fffffffu, (unsigned)__double2hiint(vb[i]) & 0x7fffffffu));
     if (xax) {
       m = __reduce_max_sync(0xffffffffu, m);
       if (lane == 0) atomicMax(&smax[l], m);
@@ -236,10 +237,33 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
       if (part == 0) atomicMax(&smax[l], m);
     }
+  } else {
+    const int width = min(32, 2 << a.log2N);  // along x: neighbouring lanes that hold entries of one stacked line
+    unsigned m = 0;
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      m = max(m, (unsigned)__double2hiint(va[i]) & 0x7fffffffu);
+      const int sl = slot_pos(i) >> a.log2N;
+      if (i < 7 && slot_pos(i + 1) >> a.log2N == sl) continue;  // uniform over the warp
+      if (xax) {
+        if (width == 32) m = __reduce_max_sync(0xffffffffu, m);
+        else
+          for (int o = 1; o < width; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+        if ((lane & (width - 1)) == 0) atomicMax(&smax[sl * kDigLines + l], m);
+      } else {
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        if (part == 0) atomicMax(&smax[sl * kDigLines + l], m);
+      }
+      m = 0;
+    }
   }
   __syncthreads();
   {
-    const int emax = max((int)(smax[l] >> 20), 1);
+    [[maybe_unused]] const int emax_l = max((int)(smax[l] >> 20), 1);
+    auto exponent = [&](int i) {
+      if constexpr (FOLD) return emax_l;
+      else return max((int)(smax[(slot_pos(i) >> a.log2N) * kDigLines + l] >> 20), 1);
+    };
     const int col = 2 * l + part;
     unsigned char* dst = dig + kg * kLbo + (col >> 3) * kSbo + (col & 7) * 16;
     uint32_t w[kDigits][4];
@@ -248,6 +272,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       long long y[2];
 #pragma unroll
       for (int k = 0; k < 2; ++k) {
+        const int emax = exponent(i + k);
         y[k] = to_fixed((uint32_t)__double2hiint(va[i + k]), (uint32_t)__double2loint(va[i + k]), emax);
         if constexpr (FOLD) {  // + or - the mirror image; the middle belongs to the sums alone
           y[k] += to_fixed((uint32_t)__double2hiint(vb[i + k]) ^ ((uint32_t)h << 31),
@@ -398,7 +423,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
     }
     return o;
   };
-  auto emit = [&](long long g, long long re, long long im, int ln, const Operands& o) {
+  auto emit = [&](long long g, long long re, long long im, int ln, const Operands& o) {  // ln: its place in smax
     const int emax = (int)(smax[ln] >> 20);
     const int ex = max(emax, 1) - 975 - (TOEP ? kDigShiftT : kDigShiftS) + a.oexp;
     double2 y = make_double2(from_fixed(re, ex), from_fixed(im, ex));
@@ -464,10 +489,10 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
     const long long dg = xax ? (NT / 128) * lstep : 2 * (NT / 16) * estep;
 #pragma unroll
     for (int it = 0; it < ITEMS; ++it) {
-      int pos = 2 * (mb * 128 + r) + h;
+      int pos = 2 * (mb * 128 + r) + h, sl = 0;
       long long line = line0 + ln;
       if constexpr (!FOLD) {
-        const int sl = r >> a.log2N;
+        sl = r >> a.log2N;
         pos = r - (sl << a.log2N);
         line += sl * kDigLines;
         g = base0 + line * lstep + pos * estep;
@@ -475,7 +500,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       const bool ok = line < nline && pos < n;
       const Operands o = fetch(g, ok);
       const longlong2 v = *reinterpret_cast<const longlong2*>(dig + r * kRowPitch + ln * 16);
-      if (ok) emit(g, v.x, v.y, ln, o);
+      if (ok) emit(g, v.x, v.y, sl * kDigLines + ln, o);
       g += dg;
       if (xax) ln += NT / 128;
       else r += NT / 16;

@@ -18,7 +18,8 @@
 // sine mode), so for n >= 255 a line is folded into its sums s_j = x_j + x_{N-j} (with x_{N/2}) and
 // differences d_j = x_j - x_{N-j}, and each half is a product of size N/2: half the work.  Shorter
 // lines are not folded; 128 / N of them are stacked into one column of 128 entries and the operator is
-// block diagonal.
+// block diagonal.  Each stacked line has its own scale: with one for the whole column a line 2^30 smaller
+// than another of its column has an error of 2e-8, and a finite line beside a non-finite one is NaN.
 //
 // Tile of a block: 128 operator rows of one half (all of it for n <= 255) times 32 columns (the real and
 // imaginary parts of 16 lines).
