@@ -341,6 +341,12 @@ long long rfnse_launch_count(void);
    limit is process-wide; no GPU memory is used up to provoke the failure.  Always RFNSE_OK. */
 int rfnse_test_fail_allocations(long long after);
 
+/* Test hook: one FP32 digit pass (the mixed form's transforms of large grids; only its solves run them
+   otherwise) along `axis`.  op 0: out = S in; 1: out = mu_a T_0 in; 2: as 1 with out in FP64.  in, out:
+   N complex FP32 device values (out complex FP64 for op 2), may not alias.  Synchronises the stream.
+   Errors: EINVAL (also when ctx has no such pass along that axis), ECUDA, ETIMEOUT. */
+int rfnse_test_digit32(rfnse_ctx* ctx, int axis, int op, const void* in, void* out);
+
 /* Measure the FMA throughput of the current device (flop/s, 2 flops per FMA) in FP64 (fp64 = 1) or
    FP32 (fp64 = 0) with independent FMA chains on 8 blocks of 256 threads per SM, timed with CUDA
    events on the legacy default stream.  Allocates and frees a small device buffer.  Used to confirm

@@ -520,6 +520,14 @@ int rfnse_toeplitz(rfnse_ctx* c, int axis, const void* in, void* out, int half) 
   return digit_status(c);
 }
 
+int rfnse_test_digit32(rfnse_ctx* c, int axis, int op, const void* in, void* out) {
+  if (!c || !in || !out || in == out || axis < 0 || axis >= c->d || op < 0 || op > 2 || !digit32_possible(c, axis))
+    return RFNSE_EINVAL;
+  RFNSE_CUDA_TRY(c, run_test_digit32(c, axis, op, (const float2*)in, out));
+  RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  return digit_status(c);
+}
+
 int rfnse_solve(rfnse_ctx* c, const double* D, const void* b, void* u, int half, int* iters, double* relres) {
   if (!c || !D || !b || !u || b == u) return RFNSE_EINVAL;
   launch_neg_i((const double2*)b, c->f, c->N, c->stream);  // f = -i b  (Sec. 3: f = [-p; q])

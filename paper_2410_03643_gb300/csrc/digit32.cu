@@ -52,6 +52,10 @@ constexpr int kOperBytes = 128 * 128 * 2;  // one digit block of the operator
 constexpr int kStage = kCtrl + 2 * kBufBytes, kOperS = (kStage + 256 * kPitch + 64 + 127) & ~127;
 constexpr int kSmem = kOperS + kOperBytes;
 static_assert(kStage % 16 == 0 && kOperS % 128 == 0, "alignment");
+// unfolded passes keep their whole operator in TMEM; its place holds the maxima and scales of up to 32 stacked lines
+// per column, for eight tiles
+constexpr int kStackMax = 32;
+static_assert(2 * 8 * kStackMax * kDigLines * 4 <= kOperBytes, "room for the stacked lines' scales");
 
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kGroup) : "memory"); }
 
@@ -94,8 +98,11 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
   const uint32_t b_empty = s0, b_dfull = s0 + 16, b_dfree = s0 + 24;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + 48);
   volatile int* s_fail = reinterpret_cast<volatile int*>(sm + 52);
-  unsigned* smax = reinterpret_cast<unsigned*>(sm + 64);  // [8][16]
-  float* sout = reinterpret_cast<float*>(sm + 576);       // [8][16]: scales of the results
+  // of eight tiles: each line's largest magnitude, and the scales of its results; [8][SL], one entry per stacked line
+  // (the operator is block diagonal, so the lines of a column need no common scale)
+  constexpr int SL = FOLD ? kDigLines : kStackMax * kDigLines;
+  unsigned* smax = reinterpret_cast<unsigned*>(sm + (FOLD ? 64 : kOperS));
+  float* sout = reinterpret_cast<float*>(sm + (FOLD ? 576 : kOperS + 8 * SL * 4));
   unsigned char* stage = sm + kStage;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int uwarp = __shfl_sync(0xffffffffu, warp, 0);
@@ -115,7 +122,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
     tc::tmem_alloc(tc::smem_addr(s_tmem), 512);
     tc::fence_before();
   }
-  if (tid < 8 * kDigLines) smax[tid] = 0;
+  for (int i = tid; i < 8 * SL; i += kNt) smax[i] = 0;
   if (FOLD) {  // digit 2 of the differences' half: K-major core matrices in shared memory
     const uint4* src = reinterpret_cast<const uint4*>(a.table + (size_t)5 * kOperBytes);
     for (int i = tid; i < kOperBytes / 16; i += kNt) {
@@ -193,30 +200,68 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
           va[i] = ln < nline && pos < n ? __ldg(in + g) : zero;
         }
       }
-      unsigned m = 0;  // the line's largest magnitude
+      // the largest magnitude of each line
+      unsigned* tmax = smax + (k & 7) * SL + l;
+      if constexpr (FOLD) {
+        unsigned m = 0;
 #pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        m = max(m, max(__float_as_uint(va[i].x) & 0x7fffffffu, __float_as_uint(va[i].y) & 0x7fffffffu));
-        if constexpr (FOLD)
+        for (int i = 0; i < 8; ++i) {
+          m = max(m, max(__float_as_uint(va[i].x) & 0x7fffffffu, __float_as_uint(va[i].y) & 0x7fffffffu));
           m = max(m, max(__float_as_uint(vb[i].x) & 0x7fffffffu, __float_as_uint(vb[i].y) & 0x7fffffffu));
+        }
+        m = max(m, __shfl_xor_sync(0xffffffffu, m, xax ? 8 : 16));
+        if (xax) {
+          m = max(m, __shfl_xor_sync(0xffffffffu, m, 4));
+          m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
+          m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
+        }
+        if (xax ? (lane & 15) == 0 : lane < 16) atomicMax(tmax, m);
+      } else {
+        const int width = min(16, 1 << a.log2N);  // along x: neighbouring lanes that hold entries of one stacked line
+        unsigned m = 0;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          m = max(m, max(__float_as_uint(va[i].x) & 0x7fffffffu, __float_as_uint(va[i].y) & 0x7fffffffu));
+          const int sl = slot_pos(i) >> a.log2N;
+          if (i < 7 && slot_pos(i + 1) >> a.log2N == sl) continue;  // uniform over the warp
+          if (xax) {
+            for (int o = 1; o < width; o <<= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if ((lane & (width - 1)) == 0) atomicMax(tmax + sl * kDigLines, m);
+          } else if (a.log2N >= 4) {  // both halves of the warp are on this stacked line
+            m = max(m, __shfl_xor_sync(0xffffffffu, m, 16));
+            if (lane < 16) atomicMax(tmax + sl * kDigLines, m);
+          } else {
+            atomicMax(tmax + sl * kDigLines, m);
+          }
+          m = 0;
+        }
       }
-      m = max(m, __shfl_xor_sync(0xffffffffu, m, xax ? 8 : 16));
-      if (xax) {
-        m = max(m, __shfl_xor_sync(0xffffffffu, m, 4));
-        m = max(m, __shfl_xor_sync(0xffffffffu, m, 2));
-        m = max(m, __shfl_xor_sync(0xffffffffu, m, 1));
-      }
-      if (xax ? (lane & 15) == 0 : lane < 16) atomicMax(&smax[(k & 7) * kDigLines + l], m);
       group_sync(1 + grp);
       // the products of this buffer's last tile (k - 2) are done; so is everything that used tile k - 4's
       // exponents, whose place tile k + 4 takes
       if (k >= 2) wait(b_empty + 8 * grp, ((k >> 1) & 1) ^ 1);
-      if (t < kDigLines) smax[((k + 4) & 7) * kDigLines + t] = 0;
-      // scale: sums of two entries below 2^(eb - 125) become at most 256; a line with an infinity or NaN is NaN
-      const unsigned mx = smax[(k & 7) * kDigLines + l];
-      const int se = min(133 - max((int)(mx >> 23), 1), 126);
-      const float f = mx >= 0x7f800000u ? __uint_as_float(0x7fc00000u) : __uint_as_float((unsigned)(se + 127) << 23);
-      if (kg == 0) sout[(k & 7) * kDigLines + l] = ldexpf(1.0f, a.oexp - se);
+      for (int i = t; i < kDigLines * a.stack; i += kGroup) smax[((k + 4) & 7) * SL + i] = 0;
+      // scale: sums of two entries below 2^(eb - 125) become at most 256; a line with an infinity or NaN is NaN (folded:
+      // through its digits; else through its results' scale, its digits zero, so that its column's other lines stay
+      // as they are)
+      auto line_scale = [&](unsigned mx, bool first, int sl) {
+        const int se = min(133 - max((int)(mx >> 23), 1), 126);
+        const bool bad = mx >= 0x7f800000u;
+        if (first) sout[(k & 7) * SL + sl * kDigLines + l] = !FOLD && bad ? __uint_as_float(0x7fc00000u) : ldexpf(1.0f, a.oexp - se);
+        return FOLD && bad ? __uint_as_float(0x7fc00000u) : __uint_as_float((unsigned)(se + 127) << 23);
+      };
+      [[maybe_unused]] float f = 0.0f;
+      if constexpr (FOLD) {
+        f = line_scale(*tmax, kg == 0, 0);
+      } else {
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int q = slot_pos(i), sl = q >> a.log2N;
+          const unsigned mx = tmax[sl * kDigLines];
+          const float fi = line_scale(mx, q == sl << a.log2N, sl);
+          va[i] = mx >= 0x7f800000u ? zero : make_float2(va[i].x * fi, va[i].y * fi);
+        }
+      }
 #pragma unroll
       for (int h = 0; h < HALVES; ++h)
 #pragma unroll
@@ -235,7 +280,8 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
               }
             }
             uint32_t d[kDigits32];
-            split2(y[0] * f, y[1] * f, d);
+            if constexpr (FOLD) split2(y[0] * f, y[1] * f, d);
+            else split2(y[0], y[1], d);
 #pragma unroll
             for (int j = 0; j < kDigits32; ++j) w[j][i >> 1] = d[j];
           }
@@ -358,7 +404,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
 #pragma unroll
         for (int i = 0; i < 4; i += 2) {
           const int ln = (c0 + i) >> 1;
-          const float f = sout[(k & 7) * kDigLines + ln];
+          const float f = sout[(k & 7) * SL + (FOLD ? 0 : (row >> a.log2N) * kDigLines) + ln];
           unsigned char* st = stage + ln * 8;
           if constexpr (FOLD && TOEP) {  // y_j = e_j + o_j, y_{N-j} = e_j - o_j
             *reinterpret_cast<float2*>(st + row * kPitch) =

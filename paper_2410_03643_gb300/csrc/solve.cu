@@ -115,6 +115,21 @@ cudaError_t run_toeplitz(rfnse_ctx* c, int axis, const double2* in, double2* out
   return solver_pass<double, double2, double2, double2, double2, F_TOEP_ACC>(c, p, axis, half ? 1 : 0, c->stream);
 }
 
+// One FP32 digit pass on its own (rfnse_test_digit32); a Toeplitz pass accumulates onto zeros.
+cudaError_t run_test_digit32(rfnse_ctx* c, int axis, int op, const float2* in, void* out) {
+  PassParams p = base_params<float>(c, axis, 0);
+  p.in = in;
+  if (op == 0) {
+    p.out = out;
+    return run_digit32<float2, double2, double2, F_DST>(c, p, axis, 0, c->stream);
+  }
+  const cudaError_t e = cudaMemsetAsync(c->wp32, 0, sizeof(float2) * c->N, c->stream);
+  if (e != cudaSuccess) return e;
+  p.acc_in = c->wp32; p.acc_out = out; p.cb = kOne;
+  if (op == 1) return run_digit32<float2, float2, float2, F_TOEP_ACC>(c, p, axis, 0, c->stream);
+  return run_digit32<float2, float2, double2, F_TOEP_ACC>(c, p, axis, 0, c->stream);
+}
+
 cudaError_t run_apply_prec(rfnse_ctx* c, const double2* v, double2* z, const double* D, int half, int precision) {
   cudaError_t e = prepare_D(c, D);
   if (e != cudaSuccess) return e;

@@ -59,7 +59,7 @@ EXPORTED = ("rfnse_default_params", "rfnse_create", "rfnse_destroy", "rfnse_last
             "rfnse_tape_forward", "rfnse_tape_backward", "rfnse_adjoint_solve", "rfnse_tban_solve",
             "rfnse_selftest_bounded_wait", "rfnse_test_fail_allocations", "rfnse_apply_prec_static",
             "rfnse_autotune", "rfnse_tuned_launches", "rfnse_batch_autotune", "rfnse_batch_set_lockstep",
-            "rfnse_batch_lockstep", "rfnse_set_arnoldi_grid", "rfnse_arnoldi_grid")
+            "rfnse_batch_lockstep", "rfnse_set_arnoldi_grid", "rfnse_arnoldi_grid", "rfnse_test_digit32")
 
 K_INSCALE, K_DST, K_LAM, K_DSCALE, K_TOEP_X, K_TOEP_ACC, K_FP32, K_DF, K_ARNOLDI = 1, 2, 4, 8, 16, 32, 256, 1024, 2048
 
@@ -148,6 +148,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     lib.rfnse_batch_set_lockstep.restype = ip
     lib.rfnse_batch_lockstep.argtypes = [vp]
     lib.rfnse_batch_lockstep.restype = ip
+    lib.rfnse_test_digit32.argtypes = [vp, ip, ip, vp, vp]
+    lib.rfnse_test_digit32.restype = ip
     lib.rfnse_test_fail_allocations.argtypes = [ctypes.c_longlong]
     lib.rfnse_test_fail_allocations.restype = ip
     if path == _build.library_path():
@@ -330,6 +332,13 @@ class Solver:
         import torch
         out = torch.empty_like(x)
         self._check(self.lib.rfnse_toeplitz(self.h, axis, _ptr(x), _ptr(out), int(half)))
+        return out
+
+    def test_digit32(self, axis: int, op: int, x):
+        """One FP32 digit pass (rfnse_test_digit32) of a complex64 tensor: op 0 S x, 1 mu T_0 x, 2 the same in FP64."""
+        import torch
+        out = torch.empty_like(x, dtype=torch.complex128 if op == 2 else x.dtype)
+        self._check(self.lib.rfnse_test_digit32(self.h, axis, op, _ptr(x), _ptr(out)))
         return out
 
     def solve(self, D, b, half: bool = False):

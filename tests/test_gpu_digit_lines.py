@@ -102,3 +102,46 @@ def test_a_line_does_not_depend_on_its_neighbours(n):
         for M, got in ((S, s.dst(axis, v)), (T, s.toeplitz(axis, v)), (T / 2, s.toeplitz(axis, v, half=True))):
             _check(M, x, e, bad, _to_lines(p, axis, got.cpu().numpy()), n[axis], 2e-15)
     s.close()
+
+
+@pytest.mark.parametrize("n", [(3, 1023, 511), (7, 511, 511), (15, 511, 255), (255, 3, 2047), (255, 7, 1023), (255, 15, 511),
+                               (63, 127, 255), (127, 255, 63)])
+def test_fp32_passes_keep_their_lines_apart(n):
+    """The same of the FP32 digit passes.  Tolerance: the sum of the leading digits is exact, the two lower ones are
+    summed in FP32 2^-11 below it, and the result is rounded once: 4 2^-24 of |M||x|."""
+    from paper_2410_03643_gb300 import Solver
+    p = _problem(n).replace(restart=2)
+    assert p.size >= 1 << 20
+    s = Solver(p, precision=1)
+    for axis in range(3):
+        if n[axis] > 255:
+            continue
+        x, e, bad = _uneven_lines(p, axis, [-60, -20, 0, 20, 60], 23 + axis)
+        x = x.astype(np.complex64)
+        v = np.empty(x.shape, dtype=np.complex64)
+        v.real, v.imag = np.ldexp(x.real, e), np.ldexp(x.imag, e)
+        for q, value in bad.items():
+            v[n[axis] // 2, q] = value
+        v = torch.from_numpy(_to_grid(p, axis, v)).cuda()
+        S, T = _matrices(p, axis)
+        x = x.astype(np.complex128)
+        for M, op in ((S, 0), (T, 1), (T, 2)):
+            y = _to_lines(p, axis, s.test_digit32(axis, op, v).cpu().numpy().astype(np.complex128))
+            _check(M, x, e, bad, y, n[axis], 4 * 2.0 ** -24)
+    s.close()
+
+
+def test_mixed_grid_with_an_axis_of_511_points():
+    """FP64 residual products as digit passes on an axis whose FP32 passes are FFT passes: two mixed steps against
+    the FP64 form, both solved to 1e-10 (1e-8 as everywhere for the mixed form)."""
+    from paper_2410_03643_gb300 import Solver
+    p = W.Problem(d=3, n=(511, 127, 127), lo=(-6.0,) * 3, hi=(6.0,) * 3, alpha=1.6, rho=1.0, dt=0.01, tol=1e-10, restart=10)
+    u0 = torch.from_numpy(W.u0_gaussian(p).reshape(-1).copy()).cuda()
+    out = []
+    for precision in (1, 0):
+        s = Solver(p, precision=precision)
+        s.set_state(u0)
+        s.run(2)
+        out.append(s.get_state()[1])
+        s.close()
+    assert float((out[0] - out[1]).norm() / out[1].norm()) < 1e-8
