@@ -126,12 +126,12 @@ TRAFFIC = {
     ("2d", "df_toep_x"): (6342912, "dcc06e68e64c"),
     ("2d", "df_toep_acc"): (8433408, "dcc06e68e64c"),
     ("3d", "arnoldi"): (1280290602, "2f0ff00eb74a"),
-    ("3d", "fp32_fused_x"): (653813546, "8c52addd920e"),
-    ("3d", "fp32_dst"): (340754232, "ead6a498f30a"),
-    ("3d", "fp32_dst_lam"): (568991829, "8c52addd920e"),
-    ("3d", "fp32_toep_acc"): (550711232, "8c52addd920e"),
-    ("3d", "df_toep_x"): (765149120, "8d048f9dab6e"),
-    ("3d", "df_toep_acc"): (749146709, "8d048f9dab6e"),
+    ("3d", "fp32_fused_x"): (654148266, "56da1858ed34"),
+    ("3d", "fp32_dst"): (340489031, "0d78b53d8ea5"),
+    ("3d", "fp32_dst_lam"): (568498218, "56da1858ed34"),
+    ("3d", "fp32_toep_acc"): (550562965, "56da1858ed34"),
+    ("3d", "df_toep_x"): (765089088, "09e1deb3ba17"),
+    ("3d", "df_toep_acc"): (749297066, "09e1deb3ba17"),
 }
 
 
