@@ -126,10 +126,10 @@ TRAFFIC = {
     ("2d", "df_toep_x"): (6342912, "dcc06e68e64c"),
     ("2d", "df_toep_acc"): (8433408, "dcc06e68e64c"),
     ("3d", "arnoldi"): (1280290602, "2f0ff00eb74a"),
-    ("3d", "fp32_fused_x"): (654148266, "56da1858ed34"),
-    ("3d", "fp32_dst"): (340489031, "0d78b53d8ea5"),
-    ("3d", "fp32_dst_lam"): (568498218, "56da1858ed34"),
-    ("3d", "fp32_toep_acc"): (550562965, "56da1858ed34"),
+    ("3d", "fp32_fused_x"): (654117717, "05851ad7710e"),
+    ("3d", "fp32_dst"): (340481464, "8fa58f83e726"),
+    ("3d", "fp32_dst_lam"): (568515456, "05851ad7710e"),
+    ("3d", "fp32_toep_acc"): (550027797, "05851ad7710e"),
     ("3d", "df_toep_x"): (765089088, "09e1deb3ba17"),
     ("3d", "df_toep_acc"): (749297066, "09e1deb3ba17"),
 }

@@ -15,7 +15,7 @@
 // digits and issue the products (alternate tiles), one group drains the accumulators and does the pointwise work,
 // which bounds the passes now.  255^3, us (bytes over time in TB/s) before and after: S 125 -> 72 (3.7), S / (w + i
 // Lambda) and S together 230 -> 191, S with the sub-solve and T_x 300 -> 217, T 227 -> 114 (3.5), T with the
-// first Gram-Schmidt dot product 236 (3.4).  The pass that also scales and stores the FP64 basis vector stays an
+// first Gram-Schmidt dot product 201 (4.0).  The pass that also scales and stores the FP64 basis vector stays an
 // FFT pass: it is bound by the FP64 products of that (148 us against 156).
 #include <cuda_fp16.h>
 #include <cmath>
@@ -59,13 +59,15 @@ static_assert(2 * 8 * kStackMax * kDigLines * 4 <= kOperBytes, "room for the sta
 
 __device__ __forceinline__ void group_sync(int id) { asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kGroup) : "memory"); }
 
-// FP32 -> FP64, exact but for subnormal values (0), by integer operations
+// FP32 -> FP64, exact, by integer operations and one FP32 product: a subnormal is scaled to the normal range first, and
+// the exponent's offset makes up for it.  (A conversion instruction for the subnormals alone, as df_f2d has, made a
+// 255^3 mixed run take 52.7 ms, this one 49.3; with subnormals set to zero by comparisons and branches it was 50.1.)
 __device__ __forceinline__ double widen(float v) {
-  const uint32_t b = __float_as_uint(v), m = b & 0x7fffffffu;
-  uint32_t hi = (m >> 3) + 0x38000000u;
-  if (m < 0x00800000u) return __hiloint2double((int)(b & 0x80000000u), 0);
-  if (m >= 0x7f800000u) hi = 0x7ff00000u | ((m & 0x7fffffu) ? 0x80000u : 0u);
-  return __hiloint2double((int)(hi | (b & 0x80000000u)), m >= 0x7f800000u ? 0 : (int)(m << 29));
+  const uint32_t m = __float_as_uint(v) & 0x7fffffffu;
+  const bool small = m < 0x00800000u;
+  const uint32_t b = __float_as_uint(v * (small ? 0x1p64f : 1.0f)), t = b & 0x7fffffffu;
+  const uint32_t offset = small ? (m ? 0x34000000u : 0u) : m >= 0x7f800000u ? 0x70000000u : 0x38000000u;
+  return __hiloint2double((int)(((t >> 3) + offset) | (b & 0x80000000u)), (int)(t << 29));
 }
 __device__ __forceinline__ void put_c(double2* p, float2 v) { *p = make_double2(widen(v.x), widen(v.y)); }
 __device__ __forceinline__ void put_c(float2* p, float2 v) { *p = v; }

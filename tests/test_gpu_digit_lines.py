@@ -145,3 +145,22 @@ def test_mixed_grid_with_an_axis_of_511_points():
         out.append(s.get_state()[1])
         s.close()
     assert float((out[0] - out[1]).norm() / out[1].norm()) < 1e-8
+
+
+def test_fp32_results_keep_their_subnormals_in_fp64():
+    """The pass that stores FP64 results stores the FP32 ones, exactly: subnormal, normal and non-finite."""
+    from paper_2410_03643_gb300 import Solver
+    p = _problem((63, 127, 255)).replace(restart=2)
+    s = Solver(p, precision=1)
+    for axis in range(3):
+        x, e, bad = _uneven_lines(p, axis, [-140, -130, 0], 41 + axis)
+        v = np.ldexp(x.real, e) + 1j * np.ldexp(x.imag, e)
+        for q, value in bad.items():
+            v[0, q] = value
+        v = torch.from_numpy(_to_grid(p, axis, v.astype(np.complex64))).cuda()
+        single = s.test_digit32(axis, 1, v).cpu().numpy().view(np.float32)
+        double = s.test_digit32(axis, 2, v).cpu().numpy().view(np.float64)
+        tiny = (single != 0) & (np.abs(single) < np.finfo(np.float32).tiny)
+        assert tiny.sum() > p.size // 10
+        assert np.array_equal(double, single.astype(np.float64), equal_nan=True)
+    s.close()
