@@ -341,6 +341,13 @@ long long rfnse_launch_count(void);
    limit is process-wide; no GPU memory is used up to provoke the failure.  Always RFNSE_OK. */
 int rfnse_test_fail_allocations(long long after);
 
+/* Test hook for the bounded waits of the digit passes: the limit of each wait of ctx's digit passes, in polls
+   (polls < 0: the default, about a second).  With 0 every such wait gives up at once, so every digit pass
+   does: it waits (with the default limit) for its own copies and products in flight, leaves its result
+   undefined and reports, and the call that ran it, or the solve (whose loops end), returns
+   RFNSE_ETIMEOUT; the context stays usable.  Drops the context's solve graphs.  Errors: EINVAL, ECUDA. */
+int rfnse_test_wait_polls(rfnse_ctx* ctx, int polls);
+
 /* Test hook: one FP32 digit pass (the mixed form's transforms of large grids; only its solves run them
    otherwise) along `axis`.  op 0: out = S in; 1: out = mu_a T_0 in; 2: as 1 with out in FP64.  in, out:
    N complex FP32 device values (out complex FP64 for op 2), may not alias.  Synchronises the stream.

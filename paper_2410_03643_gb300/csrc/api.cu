@@ -591,17 +591,19 @@ int rfnse_set_arnoldi_grid(rfnse_ctx* c, int blocks) {
   }
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
   c->coop_blocks = g;
-  for (int a = 0; a < 2; ++a)  // the cached solve graphs hold the old launch: capture them again
-    for (int h = 0; h < 2; ++h) {
-      if (c->graph_exec[a][h]) cudaGraphExecDestroy(c->graph_exec[a][h]);
-      if (c->graph[a][h]) cudaGraphDestroy(c->graph[a][h]);
-      c->graph_exec[a][h] = nullptr;
-      c->graph[a][h] = nullptr;
-    }
+  drop_solve_graphs(c);
   return RFNSE_OK;
 }
 
 int rfnse_arnoldi_grid(const rfnse_ctx* c) { return c ? c->coop_blocks : 0; }
+
+int rfnse_test_wait_polls(rfnse_ctx* c, int polls) {
+  if (!c) return RFNSE_EINVAL;
+  RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
+  c->wait_polls = polls < 0 ? kWaitPolls : polls;
+  drop_solve_graphs(c);
+  return RFNSE_OK;
+}
 
 int rfnse_test_fail_allocations(long long after) {
   g_alloc_budget.store(after < 0 ? -1 : after);

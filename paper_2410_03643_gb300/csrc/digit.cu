@@ -14,7 +14,8 @@ struct DigitArgs {
   int log2N, stack;            // log2(n + 1), lines stacked in one column
   int ca_code, cb_code;        // ca, cb as in the double-float passes (-1: any value)
   double lam_scale;            // 1 / dst_scale: lamfac holds i dst_scale / (omega + i Lambda)
-  int* err;                    // set when a bounded wait gives up
+  int polls;                   // limit of a wait
+  int *err, *loop_err;         // set when one gives up: for the host, and for the loop conditions on the device
 };
 
 // Shared memory: barriers and line exponents (of every line stacked in a column), the vector's digits, the chunk ring.  The digits are one
@@ -294,7 +295,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
 
   // ---- products: one warp issues the MMAs (all its values warp-uniform: an MMA issued from a divergent
   // branch costs 125 cycles or more of issue), another refills the chunk ring --------------------------
-  int issued = kDigStages;  // chunks requested so far (warp 1)
+  int chunks = kDigStages;  // warp 1: chunks requested so far; warp 0: chunks multiplied
   const int uwarp = __shfl_sync(0xffffffffu, warp, 0);
   if (uwarp == 0) {
     tc::fence_after();
@@ -307,8 +308,11 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
     for (int i = 0; i < kDigits && ok; ++i) {
       const uint32_t id = tc::idesc_f16(128, kDigCols * (kDigits - i));
       for (int kc = 0; kc < NK; ++kc) {
-        ok = tc::mbar_wait(b_full + 8 * st, ph);
-        if (!ok) break;
+        ok = tc::mbar_wait(b_full + 8 * st, ph, a.polls);
+        if (!ok) {
+          chunks = i * NK + kc;
+          break;
+        }
         const uint32_t kb = KB == 1 ? 0 : (uint32_t)kc / (128 / kDigChunkK);
         const uint32_t d = ud + (kb * kDigits + i) * kDigCols;
         const bool first = i == 0 && kc % (128 / kDigChunkK) == 0;
@@ -326,26 +330,43 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
       }
     }
     if (one) tc::mma_commit(b_done);
-    if (!ok && lane == 0) *s_fail = 1;
+    if (ok) chunks = NC;
+    __syncwarp();
+    if (!__all_sync(0xffffffffu, ok)) {  // the issuing lane's count is the one to go by
+      chunks = __shfl_sync(0xffffffffu, chunks, __ffs(__ballot_sync(0xffffffffu, one)) - 1);
+      *s_fail = 1;
+    }
   } else if (uwarp == 1) {
+    bool ok = true;
     for (int c = kDigStages; c < NC; ++c) {
-      if (!tc::mbar_wait(b_empty + 8 * (c % kDigStages), ((c / kDigStages) & 1) ^ 1)) {
-        if (lane == 0) *s_fail = 1;
-        break;
-      }
+      ok = tc::mbar_wait(b_empty + 8 * (c % kDigStages), ((c / kDigStages) & 1) ^ 1, a.polls);
+      if (!ok) break;
       if (lane == 0) load_chunk(c);
-      issued = c + 1;
+      chunks = c + 1;
+    }
+    __syncwarp();
+    if (!__all_sync(0xffffffffu, ok)) {
+      chunks = __shfl_sync(0xffffffffu, chunks, 0);
+      *s_fail = 1;
     }
   }
   __syncwarp();
-  if (uwarp == 0 && !tc::mbar_wait(b_done, 0) && lane == 0) *s_fail = 1;
+  if (uwarp == 0 && !tc::mbar_wait(b_done, 0, a.polls) && lane == 0) *s_fail = 1;
   __syncthreads();  // the other warps sleep here rather than poll
   tc::fence_after();
-  if (*s_fail) {  // uniform: a wait gave up; wait for the copies in flight, free TMEM and leave
-    if (tid == 32) {
-      for (int c = issued - kDigStages; c < issued; ++c)
+  if (*s_fail) {  // uniform: a wait gave up.  Wait for the products and copies in flight (they write TMEM and this
+                  // block's barriers and shared memory), free TMEM and leave
+    if (uwarp == 0) {
+      for (int c = max(chunks - kDigStages, 0); c < chunks; ++c)
+        tc::mbar_wait(b_empty + 8 * (c % kDigStages), (c / kDigStages) & 1);
+      tc::mbar_wait(b_done, 0);
+    } else if (uwarp == 1) {
+      for (int c = chunks - kDigStages; c < chunks; ++c)
         tc::mbar_wait(b_full + 8 * (c % kDigStages), (c / kDigStages) & 1);
-      if (a.err) *(volatile int*)a.err = 1;
+      if (lane == 0) {
+        *(volatile int*)a.err = 1;
+        *(volatile int*)a.loop_err = 1;
+      }
     }
     __syncthreads();
     if (warp == 0) tc::tmem_free(tmem, COLS);
@@ -569,7 +590,9 @@ cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream
   a.ca_code = coef_code(p.ca);
   a.cb_code = coef_code(p.cb);
   a.lam_scale = 1.0 / p.dst_scale;
-  a.err = &c->peek[2].err;  // pinned: written by the kernel only when a wait gives up
+  a.polls = c->wait_polls;
+  a.err = &c->peek[2].err;  // pinned
+  a.loop_err = &c->gs->err;
   const long long per = (long long)kDigLines * sh.stack;
   long long tiles;
   if (p.stride == 1) {

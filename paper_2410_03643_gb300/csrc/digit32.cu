@@ -32,7 +32,8 @@ struct Digit32Args {
   int log2N, stack;  // log2(n + 1), lines stacked in one column
   long long tiles;   // of 16 lines (columns)
   float lam_scale;   // 1 / dst_scale: lamfac holds i dst_scale / (omega + i Lambda)
-  int* err;          // set when a bounded wait gives up
+  int polls;         // limit of a wait
+  int *err, *loop_err;  // set when one gives up: for the host, and for the loop conditions on the device
 };
 
 // Warps 0-7 and 8-15 split even and odd tiles of the block, 16-23 finish them; 24 warps leave 80 registers each.
@@ -100,6 +101,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
   const uint32_t b_empty = s0, b_dfull = s0 + 16, b_dfree = s0 + 24;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + 48);
   volatile int* s_fail = reinterpret_cast<volatile int*>(sm + 52);
+  int* s_tiles = reinterpret_cast<int*>(sm + 56);  // [2]: tiles whose products each group issued
   // of eight tiles: each line's largest magnitude, and the scales of its results; [8][SL], one entry per stacked line
   // (the operator is block diagonal, so the lines of a column need no common scale)
   constexpr int SL = FOLD ? kDigLines : kStackMax * kDigLines;
@@ -151,11 +153,12 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
   __syncthreads();
   tc::fence_after();
 
-  // A wait that gives up sets s_fail, and every later one returns at once: the roles run through their tiles
-  // (on whatever data) and the block ends, reporting the failure.
+  // A wait that gives up sets s_fail, and every later one returns at once: the roles run through their tiles without
+  // further products or results, and the block ends, once the products in flight are done, reporting the failure.
   auto wait = [&](uint32_t bar, uint32_t parity) {
-    if (!*s_fail && !tc::mbar_wait(bar, parity)) *s_fail = 1;
+    if (!*s_fail && !tc::mbar_wait(bar, parity, a.polls)) *s_fail = 1;
   };
+  auto failed = [&]() { return __shfl_sync(0xffffffffu, *s_fail, 0) != 0; };  // the same in the whole warp
   const bool xax = p.stride == 1;
   const int n = p.n;
   const long long nline = xax ? p.nlines : p.stride;
@@ -177,6 +180,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
     const bool mid = FOLD && 2 * slot_pos(7) == n - 1;  // the thread's last entry is the middle of the line
     unsigned char* dst0 = sm + kCtrl + grp * kBufBytes + kg * kLbo + ((2 * l) >> 3) * kSbo + ((2 * l) & 7) * 16;
     const float2 zero = make_float2(0.0f, 0.0f);
+    [[maybe_unused]] int issued = 0;  // tiles whose products this group has issued (its first warp)
     for (int k = grp; (long long)k * gridDim.x + blockIdx.x < a.tiles; k += 2) {
       long long base0, line0;
       tile_base((long long)k * gridDim.x + blockIdx.x, base0, line0);
@@ -301,7 +305,8 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
         if (k >= 1) wait(b_dfree + 8 * (grp ^ 1), ((k - 1) >> 1) & 1);
         tc::fence_after();
         __syncwarp();
-        const bool one = tc::elect_one();
+        const bool live = !failed();
+        const bool one = tc::elect_one() && live;
         const uint32_t ud = __shfl_sync(0xffffffffu, tmem, 0);
         const uint64_t db0 = tc::smem_desc(__shfl_sync(0xffffffffu, sdig + grp * kBufBytes, 0), kLbo, kSbo);
         const uint64_t da0 = tc::smem_desc(__shfl_sync(0xffffffffu, s0 + kOperS, 0), 2048, 128);
@@ -324,8 +329,13 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
           }
         if (one) tc::mma_commit(b_empty + 8 * grp);
         if (one) tc::mma_commit(b_dfull);
+        issued += live;
         __syncwarp();
       }
+    }
+    if ((uwarp & 7) == 0) {  // nothing of this block's is in flight when it ends
+      if (issued) tc::mbar_wait(b_empty + 8 * grp, (issued - 1) & 1);
+      if (lane == 0) s_tiles[grp] = issued;
     }
   } else {
     // ---- accumulators -> results, staged by position, then the pass's pointwise work in grid order ---------------
@@ -388,44 +398,48 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
       wait(b_dfull, k & 1);
       tc::fence_after();
       __syncwarp();
+      const bool live = !failed();
       if (k) group_sync(3);  // the staged results of the tile before have been read
-      const int row = 32 * wq + lane;
+      if (live) {
+        const int row = 32 * wq + lane;
 #pragma unroll
-      for (int b = 0; b < 4; ++b) {
-        const int c0 = cg * 16 + b * 4;
-        const uint32_t ta = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)c0;
-        float D[HALVES * kDigits32][4], v[HALVES][4];
+        for (int b = 0; b < 4; ++b) {
+          const int c0 = cg * 16 + b * 4;
+          const uint32_t ta = tmem + ((uint32_t)(32 * wq) << 16) + (uint32_t)c0;
+          float D[HALVES * kDigits32][4], v[HALVES][4];
 #pragma unroll
-        for (int d = 0; d < HALVES * kDigits32; ++d) tc::tmem_ld(ta + d * kDigCols, D[d]);
-        tc::tmem_ld_wait(D);
+          for (int d = 0; d < HALVES * kDigits32; ++d) tc::tmem_ld(ta + d * kDigCols, D[d]);
+          tc::tmem_ld_wait(D);
 #pragma unroll
-        for (int h = 0; h < HALVES; ++h)
+          for (int h = 0; h < HALVES; ++h)
 #pragma unroll
-          for (int i = 0; i < 4; ++i)
-            v[h][i] = fmaf(fmaf(D[3 * h + 2][i], 0x1p-11f, D[3 * h + 1][i]), 0x1p-11f, D[3 * h][i]);
+            for (int i = 0; i < 4; ++i)
+              v[h][i] = fmaf(fmaf(D[3 * h + 2][i], 0x1p-11f, D[3 * h + 1][i]), 0x1p-11f, D[3 * h][i]);
 #pragma unroll
-        for (int i = 0; i < 4; i += 2) {
-          const int ln = (c0 + i) >> 1;
-          const float f = sout[(k & 7) * SL + (FOLD ? 0 : (row >> a.log2N) * kDigLines) + ln];
-          unsigned char* st = stage + ln * 8;
-          if constexpr (FOLD && TOEP) {  // y_j = e_j + o_j, y_{N-j} = e_j - o_j
-            *reinterpret_cast<float2*>(st + row * kPitch) =
-                make_float2((v[0][i] + v[HALVES - 1][i]) * f, (v[0][i + 1] + v[HALVES - 1][i + 1]) * f);
-            if (2 * row != n - 1)
-              *reinterpret_cast<float2*>(st + (n - 1 - row) * kPitch) =
-                  make_float2((v[0][i] - v[HALVES - 1][i]) * f, (v[0][i + 1] - v[HALVES - 1][i + 1]) * f);
-          } else {
+          for (int i = 0; i < 4; i += 2) {
+            const int ln = (c0 + i) >> 1;
+            const float f = sout[(k & 7) * SL + (FOLD ? 0 : (row >> a.log2N) * kDigLines) + ln];
+            unsigned char* st = stage + ln * 8;
+            if constexpr (FOLD && TOEP) {  // y_j = e_j + o_j, y_{N-j} = e_j - o_j
+              *reinterpret_cast<float2*>(st + row * kPitch) =
+                  make_float2((v[0][i] + v[HALVES - 1][i]) * f, (v[0][i + 1] + v[HALVES - 1][i + 1]) * f);
+              if (2 * row != n - 1)
+                *reinterpret_cast<float2*>(st + (n - 1 - row) * kPitch) =
+                    make_float2((v[0][i] - v[HALVES - 1][i]) * f, (v[0][i + 1] - v[HALVES - 1][i + 1]) * f);
+            } else {
 #pragma unroll
-            for (int h = 0; h < HALVES; ++h)
-              *reinterpret_cast<float2*>(st + row * kPitch + h * (128 * kPitch + 64)) =
-                  make_float2(v[h][i] * f, v[h][i + 1] * f);
+              for (int h = 0; h < HALVES; ++h)
+                *reinterpret_cast<float2*>(st + row * kPitch + h * (128 * kPitch + 64)) =
+                    make_float2(v[h][i] * f, v[h][i + 1] * f);
+            }
           }
         }
+        tc::fence_before();
+        __syncwarp();
+        if (lane == 0) tc::mbar_arrive(b_dfree + 8 * (k & 1));
       }
-      tc::fence_before();
-      __syncwarp();
-      if (lane == 0) tc::mbar_arrive(b_dfree + 8 * (k & 1));
       group_sync(3);
+      if (!live) continue;
 #pragma unroll
       for (int it0 = 0; it0 < ITEMS; it0 += B) {
         if (it0) fetch(it0);
@@ -461,9 +475,14 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
   }
   __syncthreads();
   if (uwarp == 16) {
+    const int tiles = s_tiles[0] + s_tiles[1];  // products are issued tile after tile, each when the one before is drained
+    if (tiles) tc::mbar_wait(b_dfull, (tiles - 1) & 1);
     tc::fence_after();
     tc::tmem_free(tmem, 512);
-    if (lane == 0 && *s_fail && a.err) *(volatile int*)a.err = 1;
+    if (lane == 0 && *s_fail) {
+      *(volatile int*)a.err = 1;
+      *(volatile int*)a.loop_err = 1;
+    }
   }
   if constexpr ((FLAGS & F_DOT0) != 0) block_sum_store(dot, p.dot_part + blockIdx.x);
 }
@@ -493,7 +512,9 @@ cudaError_t run_digit32(rfnse_ctx* c, PassParams p, int axis, int half, cudaStre
   a.log2N = p.log2L - 1;
   a.stack = sh.stack;
   a.lam_scale = (float)(1.0 / p.dst_scale);
-  a.err = &c->peek[2].err;  // pinned: written by the kernel only when a wait gives up
+  a.polls = c->wait_polls;
+  a.err = &c->peek[2].err;  // pinned
+  a.loop_err = &c->gs->err;
   p.ca_f = make_float2((float)p.ca.x, (float)p.ca.y);
   p.cb_f = make_float2((float)p.cb.x, (float)p.cb.y);
   const long long per = (long long)kDigLines * sh.stack;

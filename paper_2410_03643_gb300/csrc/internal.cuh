@@ -18,6 +18,7 @@ constexpr int kMaxM = 256;  // largest supported restart length
 // Largest grid of a last matrix-product pass that hands its <v_0, w> partials to the Arnoldi kernel
 // (every block of that kernel sums them; larger grids keep the kernel's own first sweep).
 constexpr int kDot0MaxBlocks = 4096;
+constexpr int kWaitPolls = 1 << 20;  // about a second of mbarrier polls, after which a digit pass's wait gives up
 constexpr int kNormPartMax = 4096;  // largest grid whose squared-norm partials a norm kernel sums
 
 // Number of kernels this library has launched in the process (all contexts).
@@ -311,6 +312,7 @@ struct rfnse_ctx {
   rfnse::GmresState* gs = nullptr;
   // pinned host: the statistics of a time step's solves (two), and in the third's err what digit passes report
   rfnse::GmresPeek* peek = nullptr;
+  int wait_polls = rfnse::kWaitPolls;  // the digit passes' limit (rfnse_test_wait_polls lowers it)
   int pending = 0;                   // solves of the step in flight (time_step_enqueue)
   // device-side control: cooperative Arnoldi kernel and one CUDA graph per (precision, half)
   rfnse::GridBarrier* bar = nullptr;

@@ -526,6 +526,17 @@ static cudaError_t build_solve_graph(rfnse_ctx* c, int mixed, int half) {
   return cudaSuccess;
 }
 
+// The cached solve graphs hold the launches of the old settings: the next solve captures them again.
+void drop_solve_graphs(rfnse_ctx* c) {
+  for (int a = 0; a < 2; ++a)
+    for (int h = 0; h < 2; ++h) {
+      if (c->graph_exec[a][h]) cudaGraphExecDestroy(c->graph_exec[a][h]);
+      if (c->graph[a][h]) cudaGraphDestroy(c->graph[a][h]);
+      c->graph_exec[a][h] = nullptr;
+      c->graph[a][h] = nullptr;
+    }
+}
+
 // Kernels a solve graph executed: 2 at the start, per Arnoldi step its passes and the MGS kernel, per cycle
 // the cycle start, back-substitution, update and residual kernels.
 long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk) {
@@ -1006,14 +1017,7 @@ rfnse_status autotune(rfnse_ctx* c, int reps, int force, int* n_configs, int* n_
     c->tune.clear();
     return st;
   }
-  // the cached solve graphs hold the old geometries: capture them again on the next solve
-  for (int a = 0; a < 2; ++a)
-    for (int h = 0; h < 2; ++h) {
-      if (c->graph_exec[a][h]) cudaGraphExecDestroy(c->graph_exec[a][h]);
-      if (c->graph[a][h]) cudaGraphDestroy(c->graph[a][h]);
-      c->graph_exec[a][h] = nullptr;
-      c->graph[a][h] = nullptr;
-    }
+  drop_solve_graphs(c);
   if (n_configs) *n_configs = (int)rec.size() + (tune_mgs ? 1 : 0);
   if (n_changed) *n_changed = changed;
   if (est_speedup) *est_speedup = (t_best > 0.0) ? t_dflt / t_best : 1.0;

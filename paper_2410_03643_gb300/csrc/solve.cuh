@@ -12,6 +12,7 @@ cudaError_t run_dst(rfnse_ctx* c, int axis, const double2* in, double2* out, int
 cudaError_t run_toeplitz(rfnse_ctx* c, int axis, const double2* in, double2* out, int half);
 cudaError_t run_apply_prec(rfnse_ctx* c, const double2* v, double2* z, const double* D, int half, int precision);
 cudaError_t run_test_digit32(rfnse_ctx* c, int axis, int op, const float2* in, void* out);
+void drop_solve_graphs(rfnse_ctx* c);  // after a change of what they launch
 cudaError_t run_apply_A(rfnse_ctx* c, const double2* u, double2* out, const double* D, int half);
 rfnse_status solve_block(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
                          double* relres);

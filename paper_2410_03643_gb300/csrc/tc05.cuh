@@ -2,11 +2,10 @@
 // the mbarriers and bulk copies that feed it.  Every wait is bounded.
 #pragma once
 #include <cstdint>
+#include "internal.cuh"
 
 namespace rfnse {
 namespace tc {
-
-constexpr int kWaitPolls = 1 << 20;  // about a second of mbarrier polls, then the wait gives up
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -20,9 +19,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
-// Wait until the phase of the given parity has completed; false when the wait gives up.
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
-  for (int i = 0; i < kWaitPolls; ++i) {
+// Wait until the phase of the given parity has completed; false when the wait gives up after `polls` polls.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, int polls = kWaitPolls) {
+  for (int i = 0; i < polls; ++i) {
     uint32_t ok;
     asm volatile(
         "{\n\t.reg .pred p;\n\t"

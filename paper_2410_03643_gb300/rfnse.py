@@ -59,7 +59,8 @@ EXPORTED = ("rfnse_default_params", "rfnse_create", "rfnse_destroy", "rfnse_last
             "rfnse_tape_forward", "rfnse_tape_backward", "rfnse_adjoint_solve", "rfnse_tban_solve",
             "rfnse_selftest_bounded_wait", "rfnse_test_fail_allocations", "rfnse_apply_prec_static",
             "rfnse_autotune", "rfnse_tuned_launches", "rfnse_batch_autotune", "rfnse_batch_set_lockstep",
-            "rfnse_batch_lockstep", "rfnse_set_arnoldi_grid", "rfnse_arnoldi_grid", "rfnse_test_digit32")
+            "rfnse_batch_lockstep", "rfnse_set_arnoldi_grid", "rfnse_arnoldi_grid", "rfnse_test_digit32",
+            "rfnse_test_wait_polls")
 
 K_INSCALE, K_DST, K_LAM, K_DSCALE, K_TOEP_X, K_TOEP_ACC, K_FP32, K_DF, K_ARNOLDI = 1, 2, 4, 8, 16, 32, 256, 1024, 2048
 
@@ -148,6 +149,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     lib.rfnse_batch_set_lockstep.restype = ip
     lib.rfnse_batch_lockstep.argtypes = [vp]
     lib.rfnse_batch_lockstep.restype = ip
+    lib.rfnse_test_wait_polls.argtypes = [vp, ip]
+    lib.rfnse_test_wait_polls.restype = ip
     lib.rfnse_test_digit32.argtypes = [vp, ip, ip, vp, vp]
     lib.rfnse_test_digit32.restype = ip
     lib.rfnse_test_fail_allocations.argtypes = [ctypes.c_longlong]
@@ -333,6 +336,10 @@ class Solver:
         out = torch.empty_like(x)
         self._check(self.lib.rfnse_toeplitz(self.h, axis, _ptr(x), _ptr(out), int(half)))
         return out
+
+    def test_wait_polls(self, polls: int):
+        """Limit of the digit passes' bounded waits in polls; negative: the default (rfnse_test_wait_polls)."""
+        self._check(self.lib.rfnse_test_wait_polls(self.h, int(polls)))
 
     def test_digit32(self, axis: int, op: int, x):
         """One FP32 digit pass (rfnse_test_digit32) of a complex64 tensor: op 0 S x, 1 mu T_0 x, 2 the same in FP64."""
