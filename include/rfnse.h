@@ -147,13 +147,15 @@ const char* rfnse_batch_last_error(const rfnse_batch* b);
 rfnse_ctx* rfnse_batch_context(rfnse_batch* b, int i);
 
 /* Advance every instance by nsteps time steps of the scheme (as rfnse_run).  While any instance is at
-   its first step (or has a fresh state), the instances step one after another on their streams; once
-   all are past it, one time step of the whole batch is a single CUDA graph launch: per instance its
+   its first step (or has a fresh state), each instance steps on its own stream (with device_loop all
+   instances' steps are enqueued before the first is waited for; otherwise one after another); once all
+   are past it, one time step of the whole batch is a single CUDA graph launch: per instance its
    right-hand side, its solve with device-decided loops, the update of the mixed form's cached T u
    and the rotation of its history, then a gather of every instance's statistics.  iters, relres
    (host, may be NULL): nsteps * count values, step-major ([s * count + i]).  An instance that fails
    does not stop the others: every instance takes (or fails) the step, then the call returns the first
-   failure, rfnse_batch_last_error naming its instance, without taking further steps.  Errors: EINVAL,
+   failure, rfnse_batch_last_error naming its instance, without taking further steps.  Nothing of the
+   call is left running when it returns.  Errors: EINVAL,
    ECUDA, ENOCONV (every step is still taken), ENUMERIC, ETIMEOUT. */
 int rfnse_batch_run(rfnse_batch* b, int nsteps, int* iters, double* relres);
 

@@ -566,6 +566,15 @@ int rfnse_batch_run(rfnse_batch* b, int nsteps, int* iters, double* relres) {
         if (iters) iters[(size_t)s * b->count + i] = it;
         if (relres) relres[(size_t)s * b->count + i] = rr;
       }
+      // a finished step leaves its T u (mixed form) in flight on the instance's stream: waited for before the call returns
+      for (rfnse_ctx* c : b->ctx) {
+        if (s + 1 < nsteps && fail == RFNSE_OK) break;
+        const cudaError_t e = cudaStreamSynchronize(c->stream);
+        if (e != cudaSuccess && fail == RFNSE_OK) {
+          b->err = std::string("batch step: ") + cudaGetErrorString(e);
+          fail = RFNSE_ECUDA;
+        }
+      }
       if (fail != RFNSE_OK) return fail;
       continue;
     }
