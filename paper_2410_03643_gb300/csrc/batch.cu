@@ -618,7 +618,7 @@ int rfnse_batch_run(rfnse_batch* b, int nsteps, int* iters, double* relres) {
       const GmresPeek& pk = b->h_peeks[i];
       // set-up (mixed: one kernel; FP64: D, the product passes, the sub-solve tables), the solve,
       // and (mixed) T u from the final residual
-      if (!b->lockstep) count_launch(solve_kernels(c, pk) + (c->p.precision == 1 ? 2 : 2 + c->d));
+      if (!b->lockstep) count_launch(solve_kernels(c, pk, 0) + (c->p.precision == 1 ? 2 : 2 + c->d));
       c->step += 1;
       c->iprev = (v + 1) % 3;
       c->icur = (v + 2) % 3;

@@ -23,7 +23,11 @@ constexpr int kNormPartMax = 4096;  // largest grid whose squared-norm partials 
 
 // Number of kernels this library has launched in the process (all contexts).
 extern std::atomic<long long> g_kernel_launches;
-inline void count_launch(long long k = 1) { g_kernel_launches.fetch_add(k, std::memory_order_relaxed); }
+extern thread_local long long t_kernel_launches;  // by this thread alone, captured ones included
+inline void count_launch(long long k = 1) {
+  g_kernel_launches.fetch_add(k, std::memory_order_relaxed);
+  t_kernel_launches += k;
+}
 
 // NVTX range for the span of a scope (time steps, solves, passes, the tuner), so that profilers can
 // group or select the kernels by what launched them (e.g. ncu --nvtx --nvtx-include "rfnse step/").
@@ -329,6 +333,8 @@ struct rfnse_ctx {
   cudaStream_t cap_stream = nullptr;   // private stream that captures the loop bodies
   cudaStream_t cap_stream2 = nullptr;  // private stream that captures a stand-alone solve graph
   cudaGraph_t graph[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+  // kernels of the last captured solve per [half]: before the loops, of one outer cycle, of one Arnoldi step
+  struct GraphKernels { long long start = 0, cycle = 0, step = 0; } graph_kernels[2];
   cudaGraphExec_t graph_exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
   // reverse pass (adjoint.cu): the taped forward run and its work vectors
   double2* keep_pred = nullptr;  // when set, the first time step copies its predictor here

@@ -12,6 +12,7 @@
 namespace rfnse {
 
 std::atomic<long long> g_kernel_launches{0};
+thread_local long long t_kernel_launches = 0;
 
 constexpr int kRedThreads = 256;
 

@@ -454,8 +454,15 @@ cudaError_t capture_solve(rfnse_ctx* c, int mixed, int half, cudaGraph_t g, cuda
   if ((e = cudaGraphConditionalHandleCreate(&ho, g, 0, cudaGraphCondAssignDefault)) != cudaSuccess) return fail(e);
   // solve start: x = 0, beta = ||f||, outer condition
   c->stream = s;
+  auto& kernels = c->graph_kernels[half];
+  long long counted = t_kernel_launches;
+  auto count = [&](long long* k) {
+    *k = t_kernel_launches - counted;
+    counted = t_kernel_launches;
+  };
   launch_zero(c->x, N, s);
   launch_norm_ctl(c->f, c->gs, N, c->red_blocks, c->partials, c->counter, c->bar, cfg, 0, ho, 1, s, f_part, f_n);
+  count(&kernels.start);
   if ((e = add_while_node(s, ho, &obody)) != cudaSuccess) return fail(e);
   // outer body: cycle start, inner loop, solution update, residual and the outer condition
   c->stream = bs;
@@ -490,12 +497,14 @@ cudaError_t capture_solve(rfnse_ctx* c, int mixed, int half, cudaGraph_t g, cuda
     launch_norm_ctl(c->r, c->gs, N, c->red_blocks, c->partials, c->counter, c->bar, cfg, 1, ho, 1, bs);
   }
   if ((e = cudaStreamEndCapture(bs, &obody)) != cudaSuccess) return fail(e);
+  count(&kernels.cycle);
   // inner body: one Arnoldi step
   if ((e = cudaStreamBeginCaptureToGraph(bs, ibody, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed)) !=
       cudaSuccess)
     return fail(e);
   if ((e = arnoldi_step_dev(c, half, cfg, hi, 1)) != cudaSuccess) return fail(e);
   if ((e = cudaStreamEndCapture(bs, &ibody)) != cudaSuccess) return fail(e);
+  count(&kernels.step);
   c->stream = user;
   return cudaSuccess;
 }
@@ -537,19 +546,11 @@ void drop_solve_graphs(rfnse_ctx* c) {
     }
 }
 
-// Kernels a solve graph executed: 2 at the start, per Arnoldi step its passes and the MGS kernel, per cycle
-// the cycle start, back-substitution, update and residual kernels.
-long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk) {
-  const int mixed = c->p.precision == 1 ? 1 : 0, d = c->d;
-  // a digit form makes two launches of the DST-Lambda-DST pass and of the fused x pass
-  auto digit_k = [&](int axis) {
-    return c->p.precond == 0 && c->tune.empty() && (mixed ? digit32_possible(c, axis) : digit_possible(c, axis)) ? 1 : 0;
-  };
-  const int lam_k = d > 1 ? digit_k(d - 1) : 0, fused_k = d > 1 ? digit_k(0) : 0;
-  const long long step_k = (d == 1 ? 1 : 3 * d - 2) + lam_k + fused_k + 1;
-  const long long cycle_k = mixed ? 1 + 1 + d + 1 + 1 : 1 + 1 + 1 + (d == 1 ? 1 : 2 * d - 1) + lam_k + d + 1;
-  const long long cycles = mixed ? pk.outer : (pk.it > 0 ? pk.outer + 1 : 0);
-  return 2 + step_k * pk.it + cycle_k * cycles;
+// Kernels a solve graph executed, from its statistics and the counts taken while it was captured.
+long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk, int half) {
+  const auto& k = c->graph_kernels[half];
+  const long long cycles = c->p.precision == 1 ? pk.outer : (pk.it > 0 ? pk.outer + 1 : 0);
+  return k.start + k.step * pk.it + k.cycle * cycles;
 }
 
 // Enqueue the solve of R x = f on the device loop, its statistics going to c->peek[slot]; f, x may be any
@@ -571,12 +572,13 @@ static rfnse_status solve_graph_enqueue(rfnse_ctx* c, const double* D, const dou
 }
 
 // What an enqueued solve came to, once the stream has been waited for.
-static rfnse_status solve_graph_status(rfnse_ctx* c, const GmresPeek& pk, int* iters, double* relres, int* outer_out) {
+static rfnse_status solve_graph_status(rfnse_ctx* c, const GmresPeek& pk, int half, int* iters, double* relres,
+                                       int* outer_out) {
   const int mixed = c->p.precision == 1 ? 1 : 0;
   *iters = pk.it;
   *relres = pk.relres;
   *outer_out = pk.outer;
-  count_launch(solve_kernels(c, pk));
+  count_launch(solve_kernels(c, pk, half));
   c->resid_current = mixed && pk.outer > 0;
   if (const rfnse_status sd = digit_status(c)) return sd;
   if (pk.err) { c->err = "a bounded device-side wait gave up"; return RFNSE_ETIMEOUT; }
@@ -592,7 +594,7 @@ static rfnse_status solve_graph(rfnse_ctx* c, const double* D, const double2* f,
   const rfnse_status st = solve_graph_enqueue(c, D, f, x, half, 0);
   if (st) return st;
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  return solve_graph_status(c, c->peek[0], iters, relres, outer_out);
+  return solve_graph_status(c, c->peek[0], half ? 1 : 0, iters, relres, outer_out);
 }
 
 rfnse_status solve_block(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
@@ -719,7 +721,7 @@ rfnse_status time_step_finish(rfnse_ctx* c, int* iters, double* relres) {
   int it = 0;
   for (int q = 0; q < c->pending; ++q) {
     int iq = 0, outer = 0;
-    const rfnse_status sq = solve_graph_status(c, c->peek[q], &iq, relres, &outer);
+    const rfnse_status sq = solve_graph_status(c, c->peek[q], c->step == 0 ? 1 : 0, &iq, relres, &outer);
     c->last_outer = outer;
     if (sq != RFNSE_OK && sq != RFNSE_ENOCONV) return sq;
     if (sq != RFNSE_OK) st = sq;

@@ -24,7 +24,7 @@ rfnse_status time_step_finish(rfnse_ctx* c, int* iters, double* relres);
 rfnse_status tban_solve(rfnse_ctx* c, const double* D, const double2* f, double2* x, int half, int* iters,
                         double* relres);
 // kernels one solve graph executed, from its statistics
-long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk);
+long long solve_kernels(const rfnse_ctx* c, const GmresPeek& pk, int half);
 // after the stream has been waited for: did a bounded wait of a digit pass give up since the last call?
 rfnse_status digit_status(rfnse_ctx* c);
 cudaError_t prepare_D(rfnse_ctx* c, const double* D);
