@@ -796,7 +796,9 @@ rfnse_status time_step(rfnse_ctx* c, int* iters, double* relres) {
 
 namespace {
 
-using TuneMemoKey = std::tuple<int, int, int, int, int, unsigned long long>;  // device, d, n0, n1, n2, key
+// device, d, n0, n1, n2, key, and the variant of the pass's default geometry: a mixed context below 2^20 points has no
+// digit tables and an FP64 one of the same grid has, and what is fastest without them does not decide with them
+using TuneMemoKey = std::tuple<int, int, int, int, int, unsigned long long, int>;
 std::mutex g_tune_mutex;
 std::map<TuneMemoKey, std::pair<PassGeom, PassGeom>> g_tune_memo;  // (best, default)
 std::map<TuneMemoKey, std::pair<double, double>> g_tune_times;     // (best us, default us)
@@ -893,7 +895,7 @@ rfnse_status autotune(rfnse_ctx* c, int reps, int force, int* n_configs, int* n_
   double t_best = 0.0, t_dflt = 0.0;
   rfnse_status st = RFNSE_OK;
   for (const TuneRecord& r : rec) {
-    const TuneMemoKey mk{dev, c->d, c->n[0], c->n[1], c->n[2], r.key};
+    const TuneMemoKey mk{dev, c->d, c->n[0], c->n[1], c->n[2], r.key, r.dflt.variant};
     PassGeom best = r.dflt;
     double tb = 0.0, td = 0.0;
     bool have = false;
@@ -901,13 +903,7 @@ rfnse_status autotune(rfnse_ctx* c, int reps, int force, int* n_configs, int* n_
       std::lock_guard<std::mutex> lock(g_tune_mutex);
       const auto it = g_tune_memo.find(mk);
       if (it != g_tune_memo.end()) {
-        // a choice of a context with other kernels (digit tables or none) does not apply here
-        auto same = [&](const PassGeom& g) {
-          return g.B == it->second.first.B && g.nt == it->second.first.nt && g.variant == it->second.first.variant;
-        };
-        have = same(r.dflt) || std::any_of(r.cands.begin(), r.cands.end(), same);
-      }
-      if (have) {
+        have = true;
         best = it->second.first;
         tb = g_tune_times[mk].first;
         td = g_tune_times[mk].second;
@@ -945,7 +941,7 @@ rfnse_status autotune(rfnse_ctx* c, int reps, int force, int* n_configs, int* n_
   // of the context's own basis (two sweeps and a grid-wide barrier, then the norm sweep)
   const bool tune_mgs = st == RFNSE_OK && c->N > 4096 && c->p.restart >= 1;
   if (tune_mgs) {
-    const TuneMemoKey mk{dev, -1, (int)(c->N >> 31), (int)(c->N & 0x7fffffff), 0, 0ull};
+    const TuneMemoKey mk{dev, -1, (int)(c->N >> 31), (int)(c->N & 0x7fffffff), 0, 0ull, 0};
     int best = -1;
     {
       std::lock_guard<std::mutex> lock(g_tune_mutex);
