@@ -126,12 +126,12 @@ TRAFFIC = {
     ("2d", "df_toep_x"): (6342912, "dcc06e68e64c"),
     ("2d", "df_toep_acc"): (8433408, "dcc06e68e64c"),
     ("3d", "arnoldi"): (1280290602, "2f0ff00eb74a"),
-    ("3d", "fp32_fused_x"): (653387520, "608d0ee93ff6"),
-    ("3d", "fp32_dst"): (340210958, "58e9502160e3"),
-    ("3d", "fp32_dst_lam"): (568521514, "608d0ee93ff6"),
-    ("3d", "fp32_toep_acc"): (549967253, "608d0ee93ff6"),
-    ("3d", "df_toep_x"): (765286976, "f6941d5531e0"),
-    ("3d", "df_toep_acc"): (749295530, "f6941d5531e0"),
+    ("3d", "fp32_fused_x"): (654136405, "00ca8716fabd"),
+    ("3d", "fp32_dst"): (340353095, "cf52189611c3"),
+    ("3d", "fp32_dst_lam"): (568429354, "00ca8716fabd"),
+    ("3d", "fp32_toep_acc"): (550043477, "00ca8716fabd"),
+    ("3d", "df_toep_x"): (765136512, "839b01b96df8"),
+    ("3d", "df_toep_acc"): (749329152, "839b01b96df8"),
 }
 
 

@@ -220,6 +220,9 @@ int rfnse_adjoint_solve(rfnse_ctx* ctx, const double* D, const void* g, void* la
                         double* relres);
 
 /* ---- building blocks (device pointers; used by the parity tests) ---------------------------- */
+/* In FP64 on grids of 60000 points and more (a mixed context: 2^20) their transforms run as digit products on the
+   tensor cores (axes of up to 511 points): every line on its own scale, as accurate as the FFTs; a line that holds an
+   infinity or NaN comes back as NaN.  A bounded wait inside such a pass that gives up is RFNSE_ETIMEOUT. */
 
 /* out = (D - T + iI) u, the system matrix of eq. 'equ3' (Sec. 2).  half = 1 uses mu_a/2 (first
    step).  u, out: N complex FP64 (may not alias); D: N FP64.  Errors: EINVAL, ECUDA. */
@@ -262,7 +265,7 @@ int rfnse_tban_solve(rfnse_ctx* ctx, const double* D, const void* b, void* u, in
    Either pointer may be NULL. */
 int rfnse_get_coefficients(rfnse_ctx* ctx, double* c, double* lam);
 
-/* z = F~^{-1} v exactly as rfnse_apply_prec with precision 0, but without a context and without
+/* z = F~^{-1} v as rfnse_apply_prec with precision 0 (to rounding), but without a context and without
    allocating any device memory.  (The paper has no counterpart: this is a service for callers that
    cannot call cudaMalloc -- plug-ins whose host application owns the device-memory budget,
    real-time loops that must not allocate once running, programs whose memory comes from an
@@ -298,8 +301,10 @@ int rfnse_apply_prec_static(const rfnse_params* p, const void* v, void* z, const
    the context; later launches of that configuration use it, and the context's cached solve graphs are
    dropped so that the next solve captures them again.  Choices are shared between contexts of the same
    grid on the same device unless force = 1.  The arithmetic of a line does not depend on the
-   geometry; only the order of the first MGS dot product's block partials does, so results agree with
-   an untuned context to rounding (the Arnoldi kernel's grid changes the order of its partial sums).
+   geometry, but a pass that has a form on the tensor cores (grids of 60000 points and more in FP64) may
+   be chosen as an FFT pass, which rounds differently, and the order of the first MGS dot product's block
+   partials follows the geometry, so results agree with an untuned context to rounding (the Arnoldi
+   kernel's grid changes the order of its partial sums).
    n_configs, n_changed (host, may be NULL): configurations tuned (passes, plus the Arnoldi grid) and
    how many got a geometry other than the default; est_speedup (host, may be NULL): summed default over
    summed chosen duration, one launch of each pass configuration.  Synchronises the stream.
@@ -343,12 +348,13 @@ long long rfnse_launch_count(void);
    limit is process-wide; no GPU memory is used up to provoke the failure.  Always RFNSE_OK. */
 int rfnse_test_fail_allocations(long long after);
 
-/* Test hook for the bounded waits of the digit passes: the limit of each wait of ctx's digit passes, in polls
-   (polls < 0: the default, about a second).  With 0 every such wait gives up at once, so every digit pass
-   does: it waits (with the default limit) for its own copies and products in flight, leaves its result
-   undefined and reports, and the call that ran it, or the solve (whose loops end), returns
-   RFNSE_ETIMEOUT; the context stays usable.  Drops the context's solve graphs.  Errors: EINVAL, ECUDA. */
-int rfnse_test_wait_polls(rfnse_ctx* ctx, int polls);
+/* Test hook for the bounded waits of the digit passes: in each block of such a pass of ctx, wait number `at`
+   (from 0) of the role that feeds (FP64) or drains (FP32) the products gives up without being tried, as if
+   its limit of about a second had run out (at < 0: none, the default; blocks with fewer waits run as ever).
+   The pass then waits for its own copies and products in flight, leaves its result undefined and reports,
+   and the call that ran it, or the solve (whose loops end), returns RFNSE_ETIMEOUT; the context stays
+   usable.  Drops the context's solve graphs.  Errors: EINVAL, ECUDA. */
+int rfnse_test_give_up(rfnse_ctx* ctx, int at);
 
 /* Test hook: one FP32 digit pass (the mixed form's transforms of large grids; only its solves run them
    otherwise) along `axis`.  op 0: out = S in; 1: out = mu_a T_0 in; 2: as 1 with out in FP64.  in, out:

@@ -597,10 +597,10 @@ int rfnse_set_arnoldi_grid(rfnse_ctx* c, int blocks) {
 
 int rfnse_arnoldi_grid(const rfnse_ctx* c) { return c ? c->coop_blocks : 0; }
 
-int rfnse_test_wait_polls(rfnse_ctx* c, int polls) {
+int rfnse_test_give_up(rfnse_ctx* c, int at) {
   if (!c) return RFNSE_EINVAL;
   RFNSE_CUDA_TRY(c, cudaStreamSynchronize(c->stream));
-  c->wait_polls = polls < 0 ? kWaitPolls : polls;
+  c->give_up_at = at < 0 ? -1 : at;
   drop_solve_graphs(c);
   return RFNSE_OK;
 }

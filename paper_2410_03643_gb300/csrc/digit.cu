@@ -14,13 +14,13 @@ struct DigitArgs {
   int log2N, stack;            // log2(n + 1), lines stacked in one column
   int ca_code, cb_code;        // ca, cb as in the double-float passes (-1: any value)
   double lam_scale;            // 1 / dst_scale: lamfac holds i dst_scale / (omega + i Lambda)
-  int polls;                   // limit of a wait
-  int *err, *loop_err;         // set when one gives up: for the host, and for the loop conditions on the device
+  int give_up;                 // the chunk whose request gives up untried (rfnse_test_give_up; none if negative)
+  int *err, *loop_err;         // set when a wait gives up: for the host, and for the loop conditions on the device
 };
 
-// Shared memory: barriers and line exponents (of every line stacked in a column), the vector's digits, the chunk ring.  The digits are one
-// K-major operand of 224 columns, digit j of column n at 32 j + n, because D_i .. D_6 are neighbours in
-// TMEM: for one operator digit a_i a single MMA of N = 32 (7 - i) columns forms its products with x_0 ..
+// Shared memory: barriers and line exponents (of every line stacked in a column), the vector's digits, the chunk
+// ring.  The digits are one K-major operand of 224 columns, digit j of column n at 32 j + n, because D_i .. D_6 are
+// neighbours in TMEM: for one operator digit a_i a single MMA of N = 32 (7 - i) columns forms its products with x_0 ..
 // x_{6-i}.  (An MMA costs 44 + N/2 cycles with A in shared memory, measured for N = 16..128: seven MMAs of
 // 32..224 columns per 16 entries take 751 cycles, 28 of 32 columns 1680.)  Core matrices lie 128 B (next
 // 8 columns) and 3616 B (next 8 entries) apart, so that both the threads of a strided pass (neighbouring
@@ -93,6 +93,7 @@ __device__ __forceinline__ double2 coef_times(int code, double2 c, double2 v) {
 
 // KB: K / 128 of a half; FOLD: sums and differences (two halves), else stacked whole lines.
 // 255^3, S 2000 -> 415 us, T 3870 -> 480 us (the FP64 FFT passes before, these now); 511^2, S 47 -> 24 us, T 87 -> 27.
+// An exponent for each stacked line (one for their column would not do: digit.cuh) takes 127 x 255 x 63 runs from 14.13 to 14.35 ms.
 // Nothing is saturated (255 x 255 x 63, S: ALU pipe 49%, tensor 24%, L2 17% of peak; T also FP64 23%): two blocks
 // per SM, all that TMEM holds, take turns at the integer work of the digits (4000 cycles of a tile of 16 lines
 // and one half), the products (6400), the sums (2100) and the results (3000, T 7600 with the exchange of the halves).
@@ -112,7 +113,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
   const uint32_t sring = sdig + digit_bytes<KB>();
   const uint32_t b_full = s0, b_empty = s0 + 8 * kDigStages, b_done = s0 + 16 * kDigStages;
   uint32_t* s_tmem = reinterpret_cast<uint32_t*>(sm + 96);
-  int* s_fail = reinterpret_cast<int*>(sm + 100);
+  volatile int* s_fail = reinterpret_cast<volatile int*>(sm + 100);
   unsigned* smax = reinterpret_cast<unsigned*>(sm + 128);
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
 
@@ -308,7 +309,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
     for (int i = 0; i < kDigits && ok; ++i) {
       const uint32_t id = tc::idesc_f16(128, kDigCols * (kDigits - i));
       for (int kc = 0; kc < NK; ++kc) {
-        ok = tc::mbar_wait(b_full + 8 * st, ph, a.polls);
+        ok = tc::mbar_wait(b_full + 8 * st, ph, s_fail);
         if (!ok) {
           chunks = i * NK + kc;
           break;
@@ -339,7 +340,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
   } else if (uwarp == 1) {
     bool ok = true;
     for (int c = kDigStages; c < NC; ++c) {
-      ok = tc::mbar_wait(b_empty + 8 * (c % kDigStages), ((c / kDigStages) & 1) ^ 1, a.polls);
+      ok = c != a.give_up && tc::mbar_wait(b_empty + 8 * (c % kDigStages), ((c / kDigStages) & 1) ^ 1, s_fail);
       if (!ok) break;
       if (lane == 0) load_chunk(c);
       chunks = c + 1;
@@ -351,7 +352,7 @@ __global__ void __launch_bounds__(512 * KB, KB == 1 ? 2 : 1) k_digit(const PassP
     }
   }
   __syncwarp();
-  if (uwarp == 0 && !tc::mbar_wait(b_done, 0, a.polls) && lane == 0) *s_fail = 1;
+  if (uwarp == 0 && !tc::mbar_wait(b_done, 0) && lane == 0) *s_fail = 1;
   __syncthreads();  // the other warps sleep here rather than poll
   tc::fence_after();
   if (*s_fail) {  // uniform: a wait gave up.  Wait for the products and copies in flight (they write TMEM and this
@@ -572,9 +573,10 @@ bool digit_possible(const rfnse_ctx* c, int axis) { return c->digS[axis] != null
 // FP64 FFT pass costs in proportion to the points.  A time step of the FP64 form (4 Arnoldi steps) with digit /
 // FFT passes: 127^2 0.52 / 0.40 ms, 255 x 127 0.55 / 0.43, 15 x 63 x 63 0.686 / 0.679, 255^2 0.58 / 0.60,
 // 511 x 255 0.72 / 1.04, 511^2 0.92 / 2.04, 127 x 63 x 127 1.80 / 7.01: they meet at 60000 points.
-// Mixed form: the residual products have double-float passes to beat: 255^3 860-970 against 480 us, but 511^2 33
-// against 27, and a batch of 16 grids of 127..511 points per axis took 24.9 ms with those and 25.9 with these
-// (a block here fills half an SM, so the instances' streams overlap less), hence from 2^20 points on.
+// Mixed form: the residual products have double-float passes to beat: 255^3 y, z 860 and x 973 us against 480-540 and
+// 620-630 here, 511^2 33 against 27, but a batch of 16 grids of 127..511 points per axis took 24.9 ms with those and 25.9
+// with these (a block here fills half an SM, so the instances' streams overlap less), hence from 2^20 points on.  The FP32
+// passes follow the same line; on smaller grids they have not been measured (digit32.cu takes axes of up to 255 points).
 bool digit_context(const rfnse_ctx* c) { return c->d > 1 && c->N >= (c->p.precision == 1 ? 1 << 20 : 60000); }
 
 template <int FLAGS>
@@ -590,7 +592,7 @@ cudaError_t run_digit(rfnse_ctx* c, PassParams p, int axis, int half, cudaStream
   a.ca_code = coef_code(p.ca);
   a.cb_code = coef_code(p.cb);
   a.lam_scale = 1.0 / p.dst_scale;
-  a.polls = c->wait_polls;
+  a.give_up = c->give_up_at < 0 ? -1 : kDigStages + c->give_up_at;
   a.err = &c->peek[2].err;  // pinned
   a.loop_err = &c->gs->err;
   const long long per = (long long)kDigLines * sh.stack;

@@ -42,7 +42,9 @@ constexpr int kDigChunkK = 32;    // operator entries along K per chunk: 128 row
 constexpr int kDigChunkBytes = 128 * kDigChunkK * 2;
 constexpr int kDigStages = 5;     // chunks in flight
 
-// Geometry of an axis of n points: K/128 per half, halves, lines stacked in one column.
+// Geometry of an axis of n points: K/128 per half, halves, lines stacked in one column.  1023 and 2047 points have none:
+// a tile of 128 rows and 32 columns holds kb x 7 weights x 32 columns of TMEM, 448 of its 512 columns for 511 points
+// and 896 for 1023 (a narrower tile, or rows of sums over fewer entries, has not been built).
 struct DigitShape {
   int kb, halves, stack;
 };

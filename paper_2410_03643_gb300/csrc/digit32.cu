@@ -15,7 +15,7 @@
 // digits and issue the products (alternate tiles), one group drains the accumulators and does the pointwise work,
 // which bounds the passes now.  255^3, us (bytes over time in TB/s) before and after: S 125 -> 72 (3.7), S / (w + i
 // Lambda) and S together 230 -> 191, S with the sub-solve and T_x 300 -> 217, T 227 -> 114 (3.5), T with the
-// first Gram-Schmidt dot product 201 (4.0).  The pass that also scales and stores the FP64 basis vector stays an
+// first Gram-Schmidt dot product 203 (3.9).  The pass that also scales and stores the FP64 basis vector stays an
 // FFT pass: it is bound by the FP64 products of that (148 us against 156).
 #include <cuda_fp16.h>
 #include <cmath>
@@ -32,8 +32,8 @@ struct Digit32Args {
   int log2N, stack;  // log2(n + 1), lines stacked in one column
   long long tiles;   // of 16 lines (columns)
   float lam_scale;   // 1 / dst_scale: lamfac holds i dst_scale / (omega + i Lambda)
-  int polls;         // limit of a wait
-  int *err, *loop_err;  // set when one gives up: for the host, and for the loop conditions on the device
+  int give_up;       // the block's tile whose results are given up untried (rfnse_test_give_up; none if negative)
+  int *err, *loop_err;  // set when a wait gives up: for the host, and for the loop conditions on the device
 };
 
 // Warps 0-7 and 8-15 split even and odd tiles of the block, 16-23 finish them; 24 warps leave 80 registers each.
@@ -156,7 +156,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
   // A wait that gives up sets s_fail, and every later one returns at once: the roles run through their tiles without
   // further products or results, and the block ends, once the products in flight are done, reporting the failure.
   auto wait = [&](uint32_t bar, uint32_t parity) {
-    if (!*s_fail && !tc::mbar_wait(bar, parity, a.polls)) *s_fail = 1;
+    if (!*s_fail && !tc::mbar_wait(bar, parity, s_fail)) *s_fail = 1;
   };
   auto failed = [&]() { return __shfl_sync(0xffffffffu, *s_fail, 0) != 0; };  // the same in the whole warp
   const bool xax = p.stride == 1;
@@ -395,6 +395,7 @@ __global__ void __launch_bounds__(kNt, 1) k_digit32(const PassParams p, const Di
         }
       };
       fetch(0);  // the first eight items' operands arrive while the products run
+      if (k == a.give_up) *s_fail = 1;
       wait(b_dfull, k & 1);
       tc::fence_after();
       __syncwarp();
@@ -512,7 +513,7 @@ cudaError_t run_digit32(rfnse_ctx* c, PassParams p, int axis, int half, cudaStre
   a.log2N = p.log2L - 1;
   a.stack = sh.stack;
   a.lam_scale = (float)(1.0 / p.dst_scale);
-  a.polls = c->wait_polls;
+  a.give_up = c->give_up_at;
   a.err = &c->peek[2].err;  // pinned
   a.loop_err = &c->gs->err;
   p.ca_f = make_float2((float)p.ca.x, (float)p.ca.y);

@@ -316,7 +316,7 @@ struct rfnse_ctx {
   rfnse::GmresState* gs = nullptr;
   // pinned host: the statistics of a time step's solves (two), and in the third's err what digit passes report
   rfnse::GmresPeek* peek = nullptr;
-  int wait_polls = rfnse::kWaitPolls;  // the digit passes' limit (rfnse_test_wait_polls lowers it)
+  int give_up_at = -1;               // wait of each digit-pass block that gives up untried (rfnse_test_give_up; -1: none)
   int pending = 0;                   // solves of the step in flight (time_step_enqueue)
   // device-side control: cooperative Arnoldi kernel and one CUDA graph per (precision, half)
   rfnse::GridBarrier* bar = nullptr;

@@ -49,7 +49,7 @@ cudaError_t prepare_D(rfnse_ctx* c, const double* D) {
 // w = add + a z + b (T - D) z in FP64: digit passes where they pay on every axis, otherwise circulant
 // embedding, in the mixed form with double-float FFTs (toep_df.cu) when every axis has a fixed FFT.  A
 // lock-step batch records the double-float passes (its launches cover many instances' tiles).  Digit passes
-// against the double-float ones: 255^3 480 against 860-970 us, 511^2 27 against 33 us per pass.
+// against the double-float ones: 255^3 y, z 480-540 against 860 us and x 620-630 against 973, 511^2 27 against 33 us per pass.
 cudaError_t run_matvec_fp64(rfnse_ctx* c, const double2* z, const double* D, double2* w, const double2* add,
                             double2 a, double2 b, int half, const int* skip, double* nrm_part) {
   cudaStream_t s = c->stream;

@@ -60,7 +60,7 @@ EXPORTED = ("rfnse_default_params", "rfnse_create", "rfnse_destroy", "rfnse_last
             "rfnse_selftest_bounded_wait", "rfnse_test_fail_allocations", "rfnse_apply_prec_static",
             "rfnse_autotune", "rfnse_tuned_launches", "rfnse_batch_autotune", "rfnse_batch_set_lockstep",
             "rfnse_batch_lockstep", "rfnse_set_arnoldi_grid", "rfnse_arnoldi_grid", "rfnse_test_digit32",
-            "rfnse_test_wait_polls")
+            "rfnse_test_give_up")
 
 K_INSCALE, K_DST, K_LAM, K_DSCALE, K_TOEP_X, K_TOEP_ACC, K_FP32, K_DF, K_ARNOLDI = 1, 2, 4, 8, 16, 32, 256, 1024, 2048
 
@@ -149,8 +149,8 @@ def load_library(path: Optional[str] = None) -> ctypes.CDLL:
     lib.rfnse_batch_set_lockstep.restype = ip
     lib.rfnse_batch_lockstep.argtypes = [vp]
     lib.rfnse_batch_lockstep.restype = ip
-    lib.rfnse_test_wait_polls.argtypes = [vp, ip]
-    lib.rfnse_test_wait_polls.restype = ip
+    lib.rfnse_test_give_up.argtypes = [vp, ip]
+    lib.rfnse_test_give_up.restype = ip
     lib.rfnse_test_digit32.argtypes = [vp, ip, ip, vp, vp]
     lib.rfnse_test_digit32.restype = ip
     lib.rfnse_test_fail_allocations.argtypes = [ctypes.c_longlong]
@@ -337,9 +337,9 @@ class Solver:
         self._check(self.lib.rfnse_toeplitz(self.h, axis, _ptr(x), _ptr(out), int(half)))
         return out
 
-    def test_wait_polls(self, polls: int):
-        """Limit of the digit passes' bounded waits in polls; negative: the default (rfnse_test_wait_polls)."""
-        self._check(self.lib.rfnse_test_wait_polls(self.h, int(polls)))
+    def test_give_up(self, at: int):
+        """The wait of each block of a digit pass that gives up untried; negative: none (rfnse_test_give_up)."""
+        self._check(self.lib.rfnse_test_give_up(self.h, int(at)))
 
     def test_digit32(self, axis: int, op: int, x):
         """One FP32 digit pass (rfnse_test_digit32) of a complex64 tensor: op 0 S x, 1 mu T_0 x, 2 the same in FP64."""

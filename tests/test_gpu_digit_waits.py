@@ -1,8 +1,7 @@
 """The bounded waits inside the digit passes give up: reported once, the loops end, the context stays usable.
 
-With a limit of 0 polls every wait gives up at once, on a healthy GPU: nothing hangs, the pass waits for its own copies
-and products in flight with the default limit and leaves.  Limits of a few polls give up somewhere on the way or not
-at all."""
+A wait of each block is told to give up untried, on a healthy GPU: nothing hangs, the pass waits for its own copies and
+products in flight and leaves.  The first wait gives up in every block; later ones where a block has as many."""
 import numpy as np
 import pytest
 
@@ -53,9 +52,9 @@ def test_a_wait_that_gives_up_is_reported_and_the_context_stays_usable(n, precis
         return [o.cpu().numpy() for o in out + [s.get_state()[1]]]
 
     want = everything()
-    for polls in (0, 1, 3):
-        s.test_wait_polls(polls)
-        must = polls == 0
+    for at in (0, 1, 17):
+        s.test_give_up(at)
+        must = at == 0
         for a in range(p.d):
             _gives_up(lambda: s.dst(a, u0), must)
             _gives_up(lambda: s.toeplitz(a, u0), must)
@@ -71,7 +70,7 @@ def test_a_wait_that_gives_up_is_reported_and_the_context_stays_usable(n, precis
             assert launch_count() - before < 60
         s.set_state(u0)
         _gives_up(lambda: s.run(2), must)
-    s.test_wait_polls(-1)
+    s.test_give_up(-1)
     for got, ref in zip(everything(), want):
         assert np.array_equal(got, ref)
     s.close()
@@ -85,11 +84,11 @@ def test_a_batch_names_the_instance_whose_wait_gave_up():
     u0 = torch.from_numpy(W.u0_gaussian(p).reshape(-1).copy()).cuda()
     for i in range(2):
         b.set_state(i, u0)
-    b.lib.rfnse_test_wait_polls(b.ctx[1], 0)
+    b.lib.rfnse_test_give_up(b.ctx[1], 0)
     with pytest.raises(RfnseError, match="instance 1") as e:
         b.run(1)
     assert e.value.status == RFNSE_ETIMEOUT
-    b.lib.rfnse_test_wait_polls(b.ctx[1], -1)
+    b.lib.rfnse_test_give_up(b.ctx[1], -1)
     for i in range(2):
         b.set_state(i, u0)
     b.run(3)
